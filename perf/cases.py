@@ -61,7 +61,7 @@ def listed():
          "nsrc": 16, "hb": 10.235, "tol": 2e-10, "heights": False, "phi": False},
         {"name": "mg_3d_256", "kind": "solve", "mode": "mg", "nx": 256, "ny": 256, "nz": 256,
          "nsrc": 4, "hb": 8.0, "tol": 1e-9, "heights": False, "phi": False},
-        # many maps at once: uneven sides 64 .. 1024, hbar 4 h or 8 h, 1 .. 8
+        # many maps at once: uneven sides 64 .. 1024, hbar 8 h or 12 h, 1 .. 8
         # seeds each, solved as one packed batch
         {"name": "batch_2d", "kind": "batch", "count": 12, "lo": 64, "hi": 1024, "tol": 1e-9},
         # one step of fitting a cost map to travel times at receivers: forward
@@ -171,7 +171,7 @@ def _batch_inputs(case, seed):
     out = []
     for _ in range(case["count"]):
         nx, ny = (int(v) for v in shape.integers(case["lo"], case["hi"] + 1, size=2))
-        hb, nsrc = float(shape.choice([4.0, 8.0])), int(shape.integers(1, 9))
+        hb, nsrc = float(shape.choice([8.0, 12.0])), int(shape.integers(1, 9))
         h = 1.0 / (max(nx, ny) - 1)
         out.append(((nx, ny), h, hb * h, _fourier(rng, nx, ny, h), _sources(rng, nx * ny, nsrc),
                     np.zeros(nsrc)))
@@ -290,7 +290,7 @@ def work(case):
         n = 0
         for _ in range(case["count"]):
             nx, ny = (int(v) for v in shape.integers(case["lo"], case["hi"] + 1, size=2))
-            shape.choice([4.0, 8.0]), shape.integers(1, 9)
+            shape.choice([8.0, 12.0]), shape.integers(1, 9)
             n += nx * ny
         return {"bytes": 16 * n, "flops": 100 * n}
     if kind == "train":
