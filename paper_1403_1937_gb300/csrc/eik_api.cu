@@ -14,9 +14,11 @@
 #include <vector>
 
 #include "eik_batch.h"
+#include "eik_gridsync.cuh"
 #include "eik_internal.cuh"
 #include "eik_launch.h"
 #include "eik_mixed.h"
+#include "eik_res64.h"
 
 using namespace eik;
 
@@ -56,12 +58,12 @@ constexpr int kMaxRestarts = 3;     // restarts in a row without progress
 // Kernels counted per handle (eik_kernel_stats).
 enum KernelId {
   K_SETUP64 = 0, K_SOURCES64, K_RESIDUAL64, K_PASS1_64, K_PASS2_64, K_EPILOGUE64,
-  K_SOURCE_VALUES, K_ADJ_RHS64, K_ADJ_GRAD64, K_MIXED_FIRST
+  K_SOURCE_VALUES, K_ADJ_RHS64, K_ADJ_GRAD64, K_RES64, K_MIXED_FIRST
 };
 constexpr int kMaxKernels = 32;
 const char *const kKernelNames[K_MIXED_FIRST] = {
     "setup64", "sources64", "residual64", "cg_pass1_64", "cg_pass2_64", "epilogue64",
-    "source_values", "adjoint_rhs64", "adjoint_grad64"};
+    "source_values", "adjoint_rhs64", "adjoint_grad64", "cg64_resident"};
 
 struct KernelStat {
   int64_t launches = 0, timed = 0;
@@ -88,6 +90,10 @@ struct eik_handle {
   CgState *st = nullptr;
   CgState *h_st = nullptr;     // pinned mirror
   double *part = nullptr;
+  // resident FP64 CG (grids that fit on chip), the message buffer of its
+  // grid-wide sums and, behind it, the halo inboxes of its blocks
+  Res64Plan res{};
+  unsigned long long *msg = nullptr;
   int *err = nullptr;
   int *h_err = nullptr;
   // graph of kGraphIters CG iterations for (x, r, p, q, weight)
@@ -118,6 +124,7 @@ void free_handle(eik_handle *h) {
   for (double *d : ptrs)
     if (d) cudaFree(d);
   if (h->src) cudaFree(h->src);
+  if (h->msg) cudaFree(h->msg);
   if (h->st) cudaFree(h->st);
   if (h->err) cudaFree(h->err);
   if (h->h_st) cudaFreeHost(h->h_st);
@@ -285,9 +292,24 @@ eik_status run_cg64(eik_handle *h, double *xs, const double *rhs, const double *
       stalled = 0;
     }
     last_res = std::min(last_res, now);
-    cudaGraphExec_t exec = h->profiling ? nullptr : graph_for(h, xs, weight);
+    cudaGraphExec_t exec = (h->profiling || h->res.ok) ? nullptr : graph_for(h, xs, weight);
     for (;;) {
-      if (exec) {
+      if (h->res.ok) {
+        cudaError_t e = cudaSuccess;
+        launch_k(h, K_RES64, [&] {
+          e = launch_res64(&h->res, h->g, h->sig, xs, h->r, h->p, weight, h->st, h->msg,
+                           h->msg + kSyncBytes / sizeof(*h->msg), h->stream);
+        });
+        if (e == cudaErrorCooperativeLaunchTooLarge) {
+          // fewer SMs than the device reports (a partitioned context): the
+          // two-pass form from here on; nothing has run yet
+          cudaGetLastError();
+          h->res.ok = false;
+          if (!h->profiling) exec = graph_for(h, xs, weight);
+          continue;
+        }
+        CK(e);
+      } else if (exec) {
         CK(cudaGraphLaunch(exec, h->stream));
         count_launch(h, K_PASS1_64, kGraphIters);
         count_launch(h, K_PASS2_64, kGraphIters);
@@ -315,6 +337,8 @@ eik_status run_cg64(eik_handle *h, double *xs, const double *rhs, const double *
     *iters = h->h_st->iter;
     status = (eik_status)h->h_st->status;
     if (status == EIK_ERR_BREAKDOWN) return fail(status, "CG breakdown (p.Ap <= 0)");
+    if (status == EIK_ERR_TIMEOUT)
+      return fail(status, "a device-side wait for another block's sums timed out");
     if (weight && status == EIK_OK) {
       // the recurrence met the weighted test; accept (the adjoint has no
       // componentwise true-residual form)
@@ -512,6 +536,7 @@ static eik_status create_impl(eik_handle **out, int ndim, const int64_t *dims, d
     h->cap_elem = h->num_sms * 8;
     h->nblk_stream = (int)std::min<int64_t>((n + kThreads - 1) / kThreads, h->cap_elem);
     h->nblk_part = std::max(h->nblk_stencil, h->nblk_stream);
+    size_t msg_words = 0;
 
     try {
       dalloc(&h->f, n);
@@ -526,6 +551,9 @@ static eik_status create_impl(eik_handle **out, int ndim, const int64_t *dims, d
       dalloc(&h->st, 1);
       dalloc(&h->part, 16 * (size_t)h->nblk_part);
       dalloc(&h->err, 1);
+      res64_plan(&h->res, g, h->num_sms);
+      msg_words = kSyncBytes / sizeof(*h->msg) + h->res.inbox_words;
+      dalloc(&h->msg, msg_words);
     } catch (std::bad_alloc &) {
       free_handle(h);
       return fail(EIK_ERR_OOM, "device allocation failed");
@@ -533,6 +561,7 @@ static eik_status create_impl(eik_handle **out, int ndim, const int64_t *dims, d
     CK(cudaMallocHost((void **)&h->h_st, sizeof(CgState)));
     CK(cudaMallocHost((void **)&h->h_err, sizeof(int)));
     CK(cudaMemsetAsync(h->st, 0, sizeof(CgState), h->stream));
+    CK(cudaMemsetAsync(h->msg, 0, sizeof(*h->msg) * msg_words, h->stream));
     CK(cudaMemcpyAsync(h->src, us.data(), sizeof(int64_t) * h->nsrc, cudaMemcpyHostToDevice,
                        h->stream));
     CK(cudaMemcpyAsync(h->U, uu.data(), sizeof(double) * h->nsrc, cudaMemcpyHostToDevice,
