@@ -73,6 +73,7 @@ struct MixCtl {
   int status;        // eik_status of the inner solve (EIK_OK also after a stall)
   int stalled;       // the recurrence lost positivity: the solve ended early
   int fault;         // a bounded device-side wait expired
+  float conj2;       // resident inner CG: 2 beta <p, A p_old> of the next direction
   int withhold;      // test hook: one warp never gets its first copy
   // packed batches (the single-grid passes ignore these)
   int first;         // the next pass is the inner solve's first (w = A r only)

@@ -1,34 +1,48 @@
-// Grid-wide exchange of reduction partials inside one cooperative kernel
-// (internal).  Every block publishes one or more tagged values per exchange
-// and reads those of all blocks itself, so a reduction costs one store and
-// one load round trip through L2 (no counter, no second pass over partials):
-// a value is split into two 64-bit words, each carrying the exchange's 32-bit
-// tag beside half of the value, and a reader polls both words until both tags
-// match.  Slots alternate between two sets by the tag's parity: a block can
-// be at most one exchange ahead of another, so the set it writes has been
-// read by everybody.  Polls are bounded on %globaltimer; a block that waits
-// in vain reports a fault and the kernel returns.
+// Grid-wide sums inside one cooperative kernel, and values passed from block
+// to block (internal).
+//
+// A sum: every block stores its partials in slots of its own, adds one to a
+// counter (release), waits until the counter has every block's arrival
+// (acquire, one thread), and reads all partials itself, so that all blocks add
+// the same numbers in the same order.  Measured on 152 blocks: 2,700 cycles
+// from arrival to the last partial read.  (Partials that carry a tag and are
+// polled by every block need no counter, but 152 readers polling lines that
+// eight blocks write took 5,500 to 8,000 cycles; a leader block that adds and
+// publishes took 2,600, and needs a block or warp with nothing else to do.)
+// Slots alternate between two sets by the exchange's parity: a block can be at
+// most one exchange ahead of another, so the set it writes has been read by
+// everybody.
+//
+// A value for one other block is stored as two 64-bit words, each with a
+// 32-bit tag beside half of the value, which the reader polls until both tags
+// match: no fence, no barrier.
+//
+// Every wait is bounded on %globaltimer; a block that waits in vain reports a
+// fault and the kernel returns.
 #pragma once
 
+#include <math.h>
 #include <stdint.h>
 
 namespace eik {
 
 constexpr unsigned long long kSyncWaitNs = 1000ull * 1000 * 1000;   // 1 s
 
-// Values per exchange and block that a buffer has room for.
+// Partials per exchange and block, and most blocks that take part (a warp
+// reads five slots per lane).
 constexpr int kSyncVals = 2;
+constexpr int kSyncBlocks = 160;
+// A solver's buffer: the counter in a 128-byte line, then the slots.  The
+// counter is zeroed before every launch.
+constexpr int kSyncSlot0 = 16;
+constexpr size_t kSyncBytes =
+    sizeof(unsigned long long) * (kSyncSlot0 + 2 * kSyncVals * kSyncBlocks);
 
 __device__ __forceinline__ unsigned long long sync_now() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
 }
-
-// Most blocks that take part (a warp reads five slots per lane), and the size
-// of a solver's message buffer.
-constexpr int kSyncBlocks = 160;
-constexpr size_t kSyncBytes = sizeof(unsigned long long) * 2 * kSyncVals * 2 * kSyncBlocks;
 
 // A double in two words, each with the 32-bit tag.
 __device__ __forceinline__ void tagged_put(unsigned long long *slot, unsigned tag, double x) {
@@ -63,37 +77,84 @@ __device__ __forceinline__ bool tagged_wait(const unsigned long long *slot, unsi
   }
 }
 
-__device__ __forceinline__ unsigned long long *sync_slot(unsigned long long *msg, unsigned tag,
-                                                         int v, int b, int nblk) {
-  return msg + 2 * ((size_t)((tag & 1u) * kSyncVals + v) * nblk + b);
+__device__ __forceinline__ double *sync_slot(unsigned long long *msg, unsigned tag, int v, int b) {
+  return reinterpret_cast<double *>(msg) + kSyncSlot0 + ((tag & 1u) * kSyncVals + v) * kSyncBlocks +
+         b;
 }
-
+// Block b's partial v of exchange `tag`; sync_arrive by the same thread follows.
 __device__ __forceinline__ void sync_put(unsigned long long *msg, unsigned tag, int v, int b,
-                                         int nblk, double x) {
-  tagged_put(sync_slot(msg, tag, v, b, nblk), tag, x);
+                                         double x) {
+  asm volatile("st.relaxed.gpu.global.f64 [%0], %1;" ::"l"(sync_slot(msg, tag, v, b)), "d"(x)
+               : "memory");
 }
-
-// Waits for value v of the blocks b0, b0 + 32, ... (at most N of them, those
-// below nblk); x[j] = 0 past the end.  False when the wait ran out.
-template <int N>
-__device__ __forceinline__ bool sync_wait(unsigned long long *msg, unsigned tag, int v, int b0,
-                                          int nblk, double (&x)[N]) {
-  unsigned long long t0 = 0;
-  for (unsigned spins = 1;; ++spins) {
-    bool ok = true;
-#pragma unroll
-    for (int j = 0; j < N; ++j) {
-      x[j] = 0.0;
-      if (b0 + 32 * j < nblk)
-        ok = tagged_try(sync_slot(msg, tag, v, b0 + 32 * j, nblk), tag, &x[j]) && ok;
-    }
-    if (ok) return true;
-    if ((spins & 255u) == 0u) {
-      const unsigned long long t = sync_now();
-      if (t0 == 0) t0 = t;
-      else if (t - t0 > kSyncWaitNs) return false;
+__device__ __forceinline__ void sync_arrive(unsigned long long *msg) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(msg) : "memory");
+}
+// Warp 0: waits until the counter has `target` arrivals (those of all blocks
+// in all exchanges of this launch so far).  False when the wait ran out.
+__device__ __forceinline__ bool sync_wait(unsigned long long *msg, unsigned target) {
+  int ok = 1;
+  if ((threadIdx.x & 31) == 0) {
+    unsigned long long t0 = 0;
+    for (unsigned spins = 1;; ++spins) {
+      unsigned c;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(msg) : "memory");
+      if (c >= target) break;
+      if ((spins & 255u) == 0u) {
+        const unsigned long long t = sync_now();
+        if (t0 == 0) t0 = t;
+        else if (t - t0 > kSyncWaitNs) {
+          ok = 0;
+          break;
+        }
+      }
     }
   }
+  return __shfl_sync(0xffffffffu, ok, 0) != 0;
+}
+// Warp 0, after sync_wait: partial v of the blocks lane, lane + 32, ... (0 past
+// the last).
+__device__ __forceinline__ void sync_get(unsigned long long *msg, unsigned tag, int v, int nblk,
+                                         double (&x)[kSyncBlocks / 32]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int j = 0; j < kSyncBlocks / 32; ++j) {
+    x[j] = 0.0;
+    if (lane + 32 * j < nblk)
+      asm volatile("ld.relaxed.gpu.global.f64 %0, [%1];"
+                   : "=d"(x[j])
+                   : "l"(sync_slot(msg, tag, v, lane + 32 * j))
+                   : "memory");
+  }
+}
+// Their sum over the warp, in a fixed order, in all lanes.
+__device__ __forceinline__ double sync_sum(const double (&x)[kSyncBlocks / 32]) {
+  double s = ((x[0] + x[1]) + (x[2] + x[3])) + x[4];
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
+
+// a / b for finite a >= 0 and b > 0 to about one unit in the last place (a
+// step length needs no more): a single-precision reciprocal of b's mantissa
+// and one third-order correction step, y (1 + e + e^2) with e = 1 - m y.  A
+// dependent FP64 operation takes about 90 cycles here; this has five.
+__device__ __forceinline__ double quotient(double a, double b) {
+  const int hb = __double2hiint(b);
+  const int eb = (hb >> 20) - 1023;
+  if (eb <= -1023 || eb >= 1023) return a / b;   // subnormal or near the top
+  const double m = __hiloint2double((hb & 0x000fffff) | 0x3ff00000, __double2loint(b));
+  const double y = (double)(1.0f / (float)m);
+  const double e = fma(-m, y, 1.0);
+  const double q = a * fma(y, fma(e, e, e), y);
+  // q 2^-eb: on the exponent bits unless that leaves the normal range
+  const int hq = __double2hiint(q), eq = (hq >> 20) - eb;
+  if (eq <= 0 || eq >= 2047 || (hq >> 20) == 0) return scalbn(q, -eb);
+  return __hiloint2double(hq - (eb << 20), __double2loint(q));
+}
+
+// Barrier among the first n threads of a block.
+__device__ __forceinline__ void bar_first(int id, int n) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 
 }  // namespace eik

@@ -39,6 +39,7 @@
 #include "eik_launch.h"
 #include "eik_mg.h"
 #include "eik_mixed.h"
+#include "eik_res32.h"
 
 namespace eik {
 
@@ -470,6 +471,8 @@ struct MixedState {
   int bidx = -1;
   // multigrid-preconditioned inner solve (EIK_PRECOND_MULTIGRID), else null
   MgState *mg = nullptr;
+  // resident inner CG (2D grids that fit on chip, no explicit kernel variant)
+  Res32Plan res;
   cudaGraphExec_t graph = nullptr;
   int64_t launches[8] = {0};
   // per-launch CUDA-event timing of the inner passes when profiling
@@ -623,6 +626,8 @@ eik_status mixed_create(MixedState **out, const Grid &g, const TileCount &tc, in
     g_msg = "cannot reserve shared memory for the coarse estimate";
     return EIK_ERR_CUDA;
   }
+  if (precond == EIK_PRECOND_JACOBI && tile_override == 0)
+    res32_plan(&m->res, g, m->cg, num_sms, s);
   if (precond == EIK_PRECOND_MULTIGRID) {
     const eik_status ms = mg_create(&m->mg, g, m->cg, m->px, num_sms, s);
     if (ms != EIK_OK) {
@@ -678,6 +683,7 @@ eik_status mixed_create_member(MixedState **out, const Grid &g, const TileCount 
 void mixed_destroy(MixedState *m) {
   if (!m) return;
   if (m->mg) mg_destroy(m->mg);
+  res32_destroy(&m->res);
   if (m->graph) cudaGraphExecDestroy(m->graph);
   for (auto &e : m->ev)
     if (e) cudaEventDestroy(e);
@@ -732,7 +738,7 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
   const double tol = a.opt.tol;
   const double red = (a.opt.inner_tol > 0) ? a.opt.inner_tol : kInnerReduction;
   int total = *total_io, outer = 0;
-  double best_cw = INFINITY;
+  double best_cw = INFINITY, last_cw = INFINITY;
   int stall = 0;
   eik_status result = EIK_ERR_NOT_CONVERGED;
   for (;;) {
@@ -765,10 +771,14 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
     }
     // (cw is infinite while some node of the iterate is not positive yet;
     // progress is then judged only once it is finite)
+    // a step that recovers from a bad correction (an inner solve that lost
+    // conjugacy late) counts as progress too
+    const bool recovering = cw < 0.1 * last_cw;
+    last_cw = cw;
     if (!std::isfinite(cw) || cw < 0.5 * best_cw) {
       if (std::isfinite(cw)) best_cw = cw;
       stall = 0;
-    } else if (++stall >= 2) {
+    } else if (!recovering && ++stall >= 2) {
       g_msg = "mixed refinement stopped making progress";
       break;
     }
@@ -781,8 +791,11 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
     st.alpha = 0.0;
     st.beta = 0.0;
     st.F = 0;
-    st.dF = 0;
+    // (the resident kernel moves r to its frame first; the one-pass kernels do
+    // so from their first pass's maximum)
+    st.dF = m->res.ok ? std::max(-126, std::min(126, std::ilogb(st.r_inf))) : 0;
     st.fd = st.rho_s;
+    st.conj2 = 0.f;
     st.iter = 0;
     st.done = 0;
     st.status = 0;
@@ -822,10 +835,12 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
       if (m->profile && !m->ev[0])
         for (auto &e : m->ev) MCK(cudaEventCreate(&e));
       if (m->profile) MCK(cudaEventRecord(m->ev[0], s));
-      cg32_init(m->plan, g, m->cg, m->bufs, 0, s);
+      // (the resident kernel starts from the residual's <r, r>; it has no
+      // initial pass of its own)
+      if (!m->res.ok) cg32_init(m->plan, g, m->cg, m->bufs, 0, s);
       m->launches[3]++;
       MCK(cudaGetLastError());
-      if (m->profile) {
+      if (m->profile && !m->res.ok) {
         MCK(cudaEventRecord(m->ev[1], s));
         MCK(cudaStreamSynchronize(s));
         float t = 0.f;
@@ -833,8 +848,25 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
         m->ms[3] += t;
         m->timed[3] += 1;
       }
+      int before = 0;
       for (int it = 0;; ++it) {
-        if (m->profile) {
+        if (m->res.ok) {
+          if (m->profile) MCK(cudaEventRecord(m->ev[1], s));
+          const cudaError_t e = launch_res32(&m->res, g, m->cg, m->bufs, s);
+          if (e == cudaErrorCooperativeLaunchTooLarge) {
+            // fewer SMs than the device reports (a partitioned context): the
+            // one-pass kernels from here on; nothing has run yet
+            cudaGetLastError();
+            m->res.ok = false;
+            const eik_status gs = build_graph(m, s);
+            if (gs != EIK_OK) return gs;
+            cg32_init(m->plan, g, m->cg, m->bufs, 0, s);
+            it = -1;
+            continue;
+          }
+          MCK(e);
+          if (m->profile) MCK(cudaEventRecord(m->ev[2], s));
+        } else if (m->profile) {
           // one timed iteration per host check: no launch runs past convergence
           MCK(cudaEventRecord(m->ev[1], s));
           cg32_iter(m->plan, g, m->cg, m->bufs, it & 1, s);
@@ -846,11 +878,14 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
         }
         MCK(cudaMemcpyAsync(m->h_st, m->st, sizeof(MixCtl), cudaMemcpyDeviceToHost, s));
         MCK(cudaStreamSynchronize(s));
+        const int done_now = m->h_st->iter - before;   // of the resident kernel's launch
+        before = m->h_st->iter;
+        if (m->res.ok) m->launches[4] += done_now;
         if (m->profile) {
           float t = 0.f;
           MCK(cudaEventElapsedTime(&t, m->ev[1], m->ev[2]));
           m->ms[4] += t;
-          m->timed[4] += 1;
+          m->timed[4] += m->res.ok ? done_now : 1;
         }
         if (m->h_st->done) break;
       }
@@ -902,7 +937,7 @@ eik_status mixed_solve(MixedState *m, const MixedArgs &a, int *inner_iters, int 
   m->launches[0] += 3;
   m->launches[1] += 1;
   MCK(cudaGetLastError());
-  if (!m->batch && !m->mg) {
+  if (!m->batch && !m->mg && !m->res.ok) {
     eik_status gs = build_graph(m, s);
     if (gs != EIK_OK) return gs;
   }

@@ -7,12 +7,11 @@
 // a last block that adds the partials), 22 us together on a 129^2 grid whose
 // arithmetic takes 0.3 us.  Here r, p (and x) live in registers, sigma and
 // u = sigma p in shared memory, and only the faces of a block's brick go
-// through L2; the two grid-wide sums per iteration and the face values are
-// exchanged as tagged messages (eik_gridsync.cuh), which need no fence and no
-// barrier beside them.  What is left is the FP64 pipe (two lanes per
+// through L2; the face values go as tagged messages and the two grid-wide
+// sums per iteration through one counter (eik_gridsync.cuh).  What is left is the FP64 pipe (two lanes per
 // clock and SM on this GPU: 10 instructions per node in 2D, 12 in 3D) and two
 // message round trips.  Measured per iteration (two-pass form, this one):
-// 129^2 22 us, 9 us; 733 x 517 37 us, 15 us; 120 x 97 x 85 63 us, 36 us.
+// 129^2 22 us, 10 us; 733 x 517 37 us, 14 us; 120 x 97 x 85 63 us, 35 us.
 // Larger grids, which do not fit, keep the two passes.
 //
 // Split: bricks of nearly equal size, at most one block per SM, kMinNodes
@@ -101,24 +100,6 @@ __device__ __forceinline__ double scale_down(double v, int e) {
   return __hiloint2double(ok ? hi - (e << 20) : 0, ok ? __double2loint(v) : 0);
 }
 
-// a / b for finite a >= 0 and b > 0 to about one unit in the last place (a
-// step length needs no more): a single-precision reciprocal of b's mantissa
-// and one third-order correction step, y (1 + e + e^2) with e = 1 - m y.  A
-// dependent FP64 operation takes about 90 cycles here; this has five.
-__device__ __forceinline__ double quotient(double a, double b) {
-  const int hb = __double2hiint(b);
-  const int eb = (hb >> 20) - 1023;
-  if (eb <= -1023 || eb >= 1023) return a / b;   // subnormal or near the top
-  const double m = __hiloint2double((hb & 0x000fffff) | 0x3ff00000, __double2loint(b));
-  const double y = (double)(1.0f / (float)m);
-  const double e = fma(-m, y, 1.0);
-  const double q = a * fma(y, fma(e, e, e), y);
-  // q 2^-eb: on the exponent bits unless that leaves the normal range
-  const int hq = __double2hiint(q), eq = (hq >> 20) - eb;
-  if (eq <= 0 || eq >= 2047 || (hq >> 20) == 0) return scalbn(q, -eb);
-  return __hiloint2double(hq - (eb << 20), __double2loint(q));
-}
-
 // Sum over the block in a fixed order, valid in all lanes of warp 0; the
 // return value of __syncthreads_or(flag) goes to *any.  One FP64 addition
 // keeps a quarter of the SM's FP64 lanes busy for 64 cycles, so a shuffle tree
@@ -132,7 +113,7 @@ __device__ __forceinline__ double block_sum_w0(double v, double *red, int flag, 
     const double a = (red[threadIdx.x] + red[threadIdx.x + 128]) +
                      (red[threadIdx.x + 256] + red[threadIdx.x + 384]);
     red[threadIdx.x] = a;   // read by nobody else
-    asm volatile("bar.sync 1, 128;" ::: "memory");
+    bar_first(1, 128);
     if (threadIdx.x < 32) {
       s = (a + red[threadIdx.x + 32]) + (red[threadIdx.x + 64] + red[threadIdx.x + 96]);
       for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -265,7 +246,7 @@ __global__ void __launch_bounds__(kT, 1) k_cg64_res(const Res64Args A) {
   const bool cw = A.st->stop_norm == EIK_STOP_COMPONENTWISE;
   const int max_iter = A.st->max_iter;
   int iter = A.st->iter, stop = 0, late = 0;
-  unsigned tag = A.epoch;
+  unsigned tag = A.epoch, arrivals = 0;
   __syncthreads();
 
   for (int it = 0; it < A.max_it; ++it) {
@@ -316,13 +297,16 @@ __global__ void __launch_bounds__(kT, 1) k_cg64_res(const Res64Args A) {
     double s = block_sum_w0(acc, red, late, &any);
     ++tag;
     if (tid < 32) {
-      // (a block whose halo never came says nothing, so every block stops)
-      if (tid == 0 && !any) sync_put(A.msg, tag, 0, b, nblk, s);
+      // (a block whose halo never came does not arrive, so every block stops)
+      if (tid == 0 && !any) {
+        sync_put(A.msg, tag, 0, b, s);
+        sync_arrive(A.msg);
+      }
+      arrivals += nblk;
+      const bool ok = !any && sync_wait(A.msg, arrivals);
       double v[kSyncBlocks / 32];
-      const bool ok =
-          __all_sync(0xffffffffu, !any && sync_wait(A.msg, tag, 0, tid, nblk, v));
-      double pq = ((v[0] + v[1]) + (v[2] + v[3])) + v[4];
-      for (int o = 16; o > 0; o >>= 1) pq += __shfl_xor_sync(0xffffffffu, pq, o);
+      sync_get(A.msg, tag, 0, nblk, v);
+      const double pq = sync_sum(v);
       if (tid == 0) {
         const bool pos = pq > 0.0 && finite64(pq);
         sh_val = pos ? quotient(rho, pq) : 0.0;
@@ -403,8 +387,9 @@ __global__ void __launch_bounds__(kT, 1) k_cg64_res(const Res64Args A) {
       if (half_step == 0) {
         s = block_sum_w0(acc, red, bad, &any);
         if (tid == 0) {
-          if (check) sync_put(A.msg, tag, 1, b, nblk, any ? 1.0 : 0.0);
-          sync_put(A.msg, tag, 0, b, nblk, s);
+          if (check) sync_put(A.msg, tag, 1, b, any ? 1.0 : 0.0);
+          sync_put(A.msg, tag, 0, b, s);
+          sync_arrive(A.msg);
         }
       }
     }
@@ -414,19 +399,18 @@ __global__ void __launch_bounds__(kT, 1) k_cg64_res(const Res64Args A) {
       late |= !tagged_wait(A.inbox + 2 * ((size_t)b * slots + (hi[h] >> 16)), tag, hr + h);
     if (tid < 32) {
       const double inv_rho = (rho != 0.0) ? 1.0 / rho : 0.0;
+      arrivals += nblk;
+      const bool ok = sync_wait(A.msg, arrivals);
       double v[kSyncBlocks / 32];
-      bool ok = sync_wait(A.msg, tag, 0, tid, nblk, v);
       bool fl = false;
       if (check) {
-        double f[kSyncBlocks / 32];
-        ok = sync_wait(A.msg, tag, 1, tid, nblk, f) && ok;
+        sync_get(A.msg, tag, 1, nblk, v);
 #pragma unroll
-        for (int j = 0; j < kSyncBlocks / 32; ++j) fl = fl || __double2hiint(f[j]) != 0;
+        for (int j = 0; j < kSyncBlocks / 32; ++j) fl = fl || __double2hiint(v[j]) != 0;
       }
-      ok = __all_sync(0xffffffffu, ok);
       fl = __any_sync(0xffffffffu, fl);
-      double rr = ((v[0] + v[1]) + (v[2] + v[3])) + v[4];
-      for (int o = 16; o > 0; o >>= 1) rr += __shfl_xor_sync(0xffffffffu, rr, o);
+      sync_get(A.msg, tag, 0, nblk, v);
+      const double rr = sync_sum(v);
       if (tid == 0) {
         sh_val = rr * inv_rho;
         const bool conv = cw ? (check && !fl) : rr <= nw;
@@ -568,6 +552,8 @@ cudaError_t launch_res64(Res64Plan *pl, const Grid &g, const double *sig, double
   a.epoch = pl->epoch;
   a.max_it = kRes64Iters;
   pl->epoch += 2u * kRes64Iters;
+  const cudaError_t e = cudaMemsetAsync(msg, 0, sizeof(unsigned), s);   // the arrivals
+  if (e != cudaSuccess) return e;
   void *args[] = {&a};
   return cudaLaunchCooperativeKernel((const void *)kernel_for(g.ndim, pl->per_thread),
                                      dim3(pl->nblk), dim3(kT), args, pl->smem, s);

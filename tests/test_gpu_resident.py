@@ -1,7 +1,7 @@
-"""Resident FP64 CG (csrc/eik_res64.cu) at the sizes where its split can go
-wrong, against the oracle: one block, blocks with one node in an axis, bricks
-at the limits of every nodes-per-thread instance, thin grids, grids just past
-what fits on chip (which take the two-pass kernels).
+"""The resident CG kernels (csrc/eik_res64.cu, csrc/eik_res32.cu) at the sizes
+where their splits can go wrong, against the oracle: one block, blocks with
+one node in an axis, tiles at the limits of every instance, thin grids, grids
+just past what fits on chip (which take the two-pass and one-pass kernels).
 
 Tolerance: both sides solve the same system to a componentwise residual of
 at most 1e-12.  Rows of the Jacobi-scaled operator exceed their off-diagonal
@@ -65,3 +65,38 @@ def test_resident_cg_vs_oracle(eik, dims, resident, boundary):
     else:
         S_ref, _, _, _ = cg.solve(f, dims, h, hbar, src, U, boundary=bd, tol=1e-13)
     assert np.max(np.abs(S.cpu().numpy().ravel() - S_ref)) <= 1e-8 * hbar
+
+
+# (dims, hbar / h): ragged chunks of four columns, one-row and one-column
+# tiles, every instance's tile height, level-set bands (hbar = 3 h)
+MIXED = [((2, 2), 2.0), ((3, 2), 2.0), ((5, 7), 2.0), ((2, 500), 8.0), ((500, 2), 8.0),
+         ((129, 17), 3.0), ((261, 130), 3.0), ((517, 263), 6.0), ((900, 801), 9.0),
+         ((1301, 1100), 13.0)]
+
+
+@pytest.mark.parametrize("dims,hb", MIXED)
+def test_resident_mixed_vs_oracle(eik, dims, hb):
+    """S within 1e-6, the mixed path's bound in the other tests, at tol 1e-8
+    (residual amplification below 1e4 as above, times hbar < 0.1); repeated
+    solves give the same bits, and the one-pass kernels the same S to 2e-6."""
+    import torch
+    rng = np.random.default_rng(sum(dims))
+    n = int(np.prod(dims))
+    h = 1.0 / (max(dims) - 1)
+    f = wl.fourier_field(rng, dims, h)
+    src = wl.random_sources(rng, n, min(4, n - 1))
+    U = rng.uniform(0.0, 0.01, len(src))
+    out = []
+    for variant in (0, 1):
+        opt = eik.make_options(precision="mixed", tol=1e-8, tile_override=variant)
+        hd = eik.eik_create(dims, h, hb * h, torch.from_numpy(f).cuda(), src, U, opt)
+        S, _, st = eik.eik_solve(hd)
+        if variant == 0:
+            S2, _, _ = eik.eik_solve(hd)
+            assert torch.equal(S, S2)
+        eik.eik_destroy(hd)
+        out.append(S.cpu().numpy().ravel())
+    assert np.max(np.abs(out[0] - out[1])) <= 2e-6
+    if n <= 150000:
+        sys = fd.assemble(f, dims, h, hb * h, src, U)
+        assert np.max(np.abs(out[0] - fd.solve_relative(sys))) <= 1e-6
