@@ -71,7 +71,8 @@ struct MixCtl {
   int total_iter;
   int done;          // 1: further passes return at once
   int status;        // eik_status of the inner solve (EIK_OK also after a stall)
-  int stalled;       // the recurrence lost positivity: the solve ended early
+  int stalled;       // 1: the recurrence lost positivity: the solve ended early;
+                     // 2: the residual grew too far, drop the correction
   int fault;         // a bounded device-side wait expired
   float conj2;       // resident inner CG: 2 beta <p, A p_old> of the next direction
   int withhold;      // test hook: one warp never gets its first copy

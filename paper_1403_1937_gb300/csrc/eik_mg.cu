@@ -65,7 +65,13 @@ constexpr float kOmega = 8.0f / 9.0f;   // Chebyshev-optimal single step on [1/4
 constexpr int kGraphIters = 2;          // even: the direction buffers alternate
 // an inner solve that has not met its test after this many iterations ends
 // (the refinement step then judges progress from the true residual)
-constexpr int kMaxInnerIters = 1000;
+constexpr int kMaxInnerIters = 300;
+// and so does one whose largest residual grows by this factor: the FP32
+// recurrence has come apart, and every power of ten costs a refinement step
+// to take back (measured: a 400^2 solve with hbar = 2 h whose residual had
+// grown by 1e14 and 1e18 took 18 steps, or all 30, to return).  Its correction
+// is dropped (MixCtl.stalled = 2).
+constexpr float kMaxGrowth = 1e4f;
 thread_local std::string g_msg = "no error";
 
 enum { kW = 0, kE = 1, kS = 2, kN = 3, kB = 4, kT = 5, kDirs = 6 };
@@ -76,7 +82,9 @@ struct MgLevel {
   float *ia = nullptr;           // 1 / a (0 on nodes with no unknowns)
   float *c = nullptr;            // kDirs x m row-relative coefficients (W, E, S, N, B, T)
   int *k = nullptr;
-  float *g = nullptr, *y = nullptr;
+  // restricted residual, its pre-smoothed correction omega g / a (written
+  // beside it, so that neighbours read one array instead of two), correction
+  float *g = nullptr, *yp = nullptr, *y = nullptr;
 };
 
 struct MgCtl {
@@ -84,6 +92,7 @@ struct MgCtl {
   double alpha, beta;
   int iter, max_iter, done, status, stalled, mode, first, kmin;
   float thresh, theta;
+  float r_limit;     // the inner solve ends where max |r| grows past this
   unsigned int counter[4];
 };
 
@@ -105,64 +114,22 @@ __device__ __forceinline__ float p2f(int e) {
   return (e < -126) ? 0.f : __int_as_float((e + 127) << 23);
 }
 
-// Grid-stride loops over the rows (y, z) of a level (blockIdx.y) and its
-// columns x: no 64-bit division per node.
-#define MG_ROWS(ny_, nz_)                                              \
-  for (int rr = blockIdx.y; rr < (ny_) * (nz_); rr += gridDim.y)      \
+// Grid-stride loops over the rows (y, z) of a level and its columns x: no
+// 64-bit division per node.  Blocks are as wide as the row needs (grid2), so
+// that short rows leave no threads idle.
+#define MG_ROWS(ny_, nz_)                                                           \
+  for (int rr = blockIdx.y * blockDim.y + threadIdx.y; rr < (ny_) * (nz_);          \
+       rr += gridDim.y * blockDim.y)                                                \
     for (int y = rr % (ny_), z = rr / (ny_), once_ = 1; once_; once_ = 0)
 #define MG_COLS(nx_) \
   for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < (nx_); x += gridDim.x * blockDim.x)
 
-// Level-0 off-diagonal sum  sig_i sum_j omega_ij sig_j 2^(k_i - k_j) v(j)
-// for the node (x, y, z); v(j, xj, yj, zj) gives the vector at pitched
-// index j.  The exponent is looked up only where the neighbour lies in
-// another cell.  Edge weights: the product of the face factors of the other
-// axes (Sec. 6 with zero-flux faces, half cells on the faces).
 // Linear index of (x, y, z) on a level of pitch nx and ny rows per plane
 // (DIM = 2: z is 0).
 template <int DIM>
 __device__ __forceinline__ int64_t lin(int x, int y, int z, int nx, int ny) {
   if constexpr (DIM == 3) return x + (int64_t)nx * (y + (int64_t)ny * z);
   else return x + (int64_t)nx * y;
-}
-
-template <int DIM, class V>
-__device__ __forceinline__ float nb0(const Grid &g, const CellGrid &cg, int px,
-                                     const float *__restrict__ s32, const int *__restrict__ kx,
-                                     int x, int y, int z, int ki, V v) {
-  float acc = 0.f;
-  const int mask = cg.B - 1;
-  const float hx = face(x, g.nx, g.boundary), hy = face(y, g.ny, g.boundary);
-  const float hz = (DIM == 3) ? facez(g, z) : 1.f;
-  const int64_t i = lin<DIM>(x, y, z, px, g.ny);
-  if (x > 0) {
-    const float f = ((x & mask) == 0) ? p2f(ki - kx_at(cg, x - 1, y, z, kx)) : 1.f;
-    acc = fmaf(hy * hz * s32[i - 1] * f, v(i - 1, x - 1, y, z), acc);
-  }
-  if (x + 1 < g.nx) {
-    const float f = (((x + 1) & mask) == 0) ? p2f(ki - kx_at(cg, x + 1, y, z, kx)) : 1.f;
-    acc = fmaf(hy * hz * s32[i + 1] * f, v(i + 1, x + 1, y, z), acc);
-  }
-  if (y > 0) {
-    const float f = ((y & mask) == 0) ? p2f(ki - kx_at(cg, x, y - 1, z, kx)) : 1.f;
-    acc = fmaf(hx * hz * s32[i - px] * f, v(i - px, x, y - 1, z), acc);
-  }
-  if (y + 1 < g.ny) {
-    const float f = (((y + 1) & mask) == 0) ? p2f(ki - kx_at(cg, x, y + 1, z, kx)) : 1.f;
-    acc = fmaf(hx * hz * s32[i + px] * f, v(i + px, x, y + 1, z), acc);
-  }
-  if constexpr (DIM == 3) {
-    const int64_t pz = (int64_t)px * g.ny;
-    if (z > 0) {
-      const float f = ((z & mask) == 0) ? p2f(ki - kx_at(cg, x, y, z - 1, kx)) : 1.f;
-      acc = fmaf(hx * hy * s32[i - pz] * f, v(i - pz, x, y, z - 1), acc);
-    }
-    if (z + 1 < g.nz) {
-      const float f = (((z + 1) & mask) == 0) ? p2f(ki - kx_at(cg, x, y, z + 1, kx)) : 1.f;
-      acc = fmaf(hx * hy * s32[i + pz] * f, v(i + pz, x, y, z + 1), acc);
-    }
-  }
-  return s32[i] * acc;
 }
 
 // Coarse-level operator (A u)_t for node (x, y, z) of a level; u(j, xj, yj,
@@ -361,37 +328,11 @@ __global__ void k_mg_coarsen(MgLevel F, MgLevel C) {
 }
 
 // ------------------------------------------------------------- V-cycle
-// Level 0 down: y = omega r, t = r - A y, g1 = sum over the box of w_i t_i.
-template <int DIM>
-__global__ void k_mg_down0(Grid g, CellGrid cg, int px, const float *__restrict__ s32,
-                           const int *__restrict__ kx, const float *__restrict__ w,
-                           const float *__restrict__ r, MgLevel L1, const MgCtl *ctl) {
-  if (ctl->done) return;
-  auto rv = [&](int64_t j, int, int, int) { return r[j]; };
-  MG_ROWS(L1.ny, L1.nz) MG_COLS(L1.nx) {
-    float sum = 0.f;
-    const int zt = (DIM == 3) ? min(2 * z + 1, g.nz - 1) : 0;
-    for (int cz = 2 * z; cz <= zt; ++cz)
-      for (int cy = 2 * y; cy <= min(2 * y + 1, g.ny - 1); ++cy)
-        for (int cx = 2 * x; cx <= min(2 * x + 1, g.nx - 1); ++cx) {
-          const int64_t i = lin<DIM>(cx, cy, cz, px, g.ny);
-          const float wi = w[i];
-          if (wi == 0.f) continue;
-          const int ki = kx_at(cg, cx, cy, cz, kx);
-          const float off = nb0<DIM>(g, cg, px, s32, kx, cx, cy, cz, ki, rv);
-          // (A (omega r))_i = omega (r_i - off)
-          const float ti = r[i] - kOmega * (r[i] - off);
-          sum = fmaf(wi, ti, sum);
-        }
-    L1.g[x + (int64_t)L1.nx * rr] = sum;
-  }
-}
-
-// Level l down (l >= 1) at coarse node (x, y, z): y = omega g / a on the
-// box, t = g - A y, restricted to level l + 1.
+// Level l down (l >= 1) at coarse node (x, y, z): t = g - A yp on the box,
+// restricted to level l + 1, and that level's pre-smoothed correction.
 template <int DIM>
 __device__ __forceinline__ void down_node(const MgLevel &F, const MgLevel &C, int x, int y, int z) {
-  auto yv = [&](int64_t j, int, int, int) { return kOmega * F.g[j] * F.ia[j]; };
+  auto yv = [&](int64_t j, int, int, int) { return F.yp[j]; };
   const int64_t t = lin<DIM>(x, y, z, C.nx, C.ny);
   const int kc = C.k[t];
   float sum = 0.f;
@@ -407,6 +348,7 @@ __device__ __forceinline__ void down_node(const MgLevel &F, const MgLevel &C, in
         }
   }
   C.g[t] = sum;
+  C.yp[t] = kOmega * sum * C.ia[t];
 }
 
 template <int DIM>
@@ -415,8 +357,9 @@ __global__ void k_mg_down(MgLevel F, MgLevel C, const MgCtl *ctl) {
   MG_ROWS(C.ny, C.nz) MG_COLS(C.nx) down_node<DIM>(F, C, x, y, z);
 }
 
-// Level l up (l >= 1) at node (x, y, z): u = omega g / a + y(parent);
-// y = u + omega (g - A u) / a.
+// Level l up (l >= 1) at node (x, y, z): u = yp + y(parent);
+// y = u + omega (g - A u) / a.  (Coefficients towards nodes with no unknowns
+// are 0, so their parents' values do not enter.)
 template <int DIM>
 __device__ __forceinline__ void up_node(const MgLevel &F, const MgLevel &C, int x, int y, int z) {
   const int64_t t = lin<DIM>(x, y, z, F.nx, F.ny);
@@ -425,8 +368,7 @@ __device__ __forceinline__ void up_node(const MgLevel &F, const MgLevel &C, int 
     return;
   }
   auto uat = [&](int64_t j, int xj, int yj, int zj) {
-    const float par = (F.a[j] >= 0.f) ? C.y[lin<DIM>(xj >> 1, yj >> 1, zj >> 1, C.nx, C.ny)] : 0.f;
-    return fmaf(kOmega * F.g[j], F.ia[j], par);
+    return F.yp[j] + C.y[lin<DIM>(xj >> 1, yj >> 1, zj >> 1, C.nx, C.ny)];
   };
   const float ut = uat(t, x, y, z);
   const float Au = apply_l<DIM>(F, x, y, z, uat);
@@ -473,62 +415,175 @@ __global__ void __launch_bounds__(kTailThreads) k_mg_tail(MgTail T, const MgCtl 
   }
 }
 
-// ------------------------------------------------------------- PCG passes
-// Inner-product weight 2^(-2 (k - kmin)); 0 past the FP32 range, where a
-// term is below 2^-126 of the nearest ones.  Per-thread sums are FP32, the
-// block and grid sums FP64.
-__device__ __forceinline__ float wdot(int k, int kmin) { return p2f(2 * (kmin - k)); }
+// ------------------------------------------------ level-0 passes (tiled)
+// The three level-0 passes of an iteration share one shape: form a vector v
+// from one to three arrays, apply the operator A to it, and combine.  Each
+// node's u = sigma v is formed once and its neighbours' come from registers
+// (z in 3D, y in 2D), a shuffle (x) and shared memory (y in 3D); gathering
+// them per node, as these passes did before, formed every u five or seven
+// times from up to four loads each and left them bound by load latency
+// (256^3: 1.19 ms an iteration for the three, 0.42 ms now; 2048^2: 163 us, 83 us).
+//   down (kDown): v = r;                g1 = sum over the box of w (r - omega (r - A' v)),
+//   up   (kUp):   v = omega r + w y1,   z = v + omega (r - A v), <r, z>,
+//   dir  (kDir):  v = z + beta p_old,   p = v, q = A v, <p, q>.
+// Tiles are 128 columns (four per lane) x 8 rows per warp in 2D, x 16 rows x
+// up to 16 planes per block in 3D: with cells of at least 16 nodes a tile
+// lies in one cell row and layer, so a lane has one cell exponent, and the
+// factors 2^(k_i - k_j) differ from 1 at the tile's rim only.
+enum { kDown = 0, kUp = 1, kDir = 2 };
 
-__device__ __forceinline__ int block_id() { return blockIdx.y * gridDim.x + blockIdx.x; }
-__device__ __forceinline__ int block_count() { return gridDim.x * gridDim.y; }
+struct Mg0 {
+  Grid g;
+  CellGrid cg;
+  int px;
+  const float *s32;
+  const int *kx;
+  const float *w, *r, *z, *p_old;
+  float *out, *out2;    // up: z; dir: p_new, q; down: the level-1 residual
+  const float *y1;      // level-1 correction
+  int nx1, ny1;         // level-1 extents
+  const float *ia1;     // level-1 inverse diagonal (down: out2 = yp)
+};
 
-// Last-block-done over a 2D grid (all gridDim.x * gridDim.y blocks): true in
-// the block that arrives last, after every block has written its partials.
-__device__ __forceinline__ bool last_block_2d(unsigned int *ticket, int *sh_flag) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    const unsigned int t = atomicAdd(ticket, 1u);
-    *sh_flag = (t == (unsigned int)block_count() - 1u);
-  }
-  __syncthreads();
-  const bool last = *sh_flag != 0;
-  if (last) __threadfence();
-  return last;
+__device__ __forceinline__ float4 ld4g(const float *p) {
+  return __ldg(reinterpret_cast<const float4 *>(p));
+}
+__device__ __forceinline__ float f4(const float4 &v, int i) {
+  return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w;
 }
 
-// Level 0 up: u = omega r + w y1(parent), z = u + omega (r - A u); rho = <r, z>.
-template <int DIM>
-__global__ void __launch_bounds__(kThreads)
-k_mg_up0(Grid g, CellGrid cg, int px, const float *__restrict__ s32, const int *__restrict__ kx,
-         const float *__restrict__ w, const float *__restrict__ r, MgLevel L1,
-         float *__restrict__ zv, MgCtl *ctl, double *part) {
+// One row of a tile at pitched offset o: sigma, v and the arrays that the
+// output needs later (a: r in kDown and kUp).  y1x/y1y: the parents'
+// corrections of the lane's two column pairs.
+struct Row0 {
+  float4 s, v, a, w;
+};
+template <int MODE>
+__device__ __forceinline__ Row0 row0_load(const Mg0 &A, int64_t o, bool in, float y1x, float y1y,
+                                          float beta, bool first) {
+  Row0 R;
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  R.s = R.v = R.a = R.w = zero;
+  if (!in) return R;
+  R.s = ld4g(A.s32 + o);
+  if (MODE == kDown) {
+    R.a = R.v = ld4g(A.r + o);
+  } else if (MODE == kUp) {
+    R.a = ld4g(A.r + o);
+    const float4 w = ld4g(A.w + o);
+    R.v = make_float4(fmaf(w.x, y1x, kOmega * R.a.x), fmaf(w.y, y1x, kOmega * R.a.y),
+                      fmaf(w.z, y1y, kOmega * R.a.z), fmaf(w.w, y1y, kOmega * R.a.w));
+  } else {
+    R.v = ld4g(A.z + o);
+    if (!first) {
+      const float4 p = ld4g(A.p_old + o);
+      R.v = make_float4(fmaf(beta, p.x, R.v.x), fmaf(beta, p.y, R.v.y), fmaf(beta, p.z, R.v.z),
+                        fmaf(beta, p.w, R.v.w));
+    }
+  }
+  return R;
+}
+// u = sigma v of one node beside the tile (column x0 - 1 or x0 + 128).
+template <int MODE>
+__device__ __forceinline__ float rim0(const Mg0 &A, int64_t o, bool in, float y1, float beta,
+                                      bool first) {
+  if (!in) return 0.f;
+  const float s = __ldg(A.s32 + o);
+  if (MODE == kDown) return s * __ldg(A.r + o);
+  if (MODE == kUp) return s * fmaf(__ldg(A.w + o), y1, kOmega * __ldg(A.r + o));
+  return s * (first ? __ldg(A.z + o) : fmaf(beta, __ldg(A.p_old + o), __ldg(A.z + o)));
+}
+__device__ __forceinline__ float4 mul4f(const float4 &a, const float4 &b) {
+  return make_float4(a.x * b.x, a.y * b.y, a.z * b.z, a.w * b.w);
+}
+
+// Output of one row: off[i] = sigma_i sum of the neighbours' u.  Returns the
+// lane's dot terms (times the weight wd) of kUp and kDir; kDown adds w t to
+// the box sums c0, c1.
+template <int MODE>
+__device__ __forceinline__ float row0_out(const Mg0 &A, int64_t o, const Row0 &R,
+                                          const float (&off)[4], float wd, float &c0, float &c1) {
+  if (MODE == kDown) {
+    const float4 w = ld4g(A.w + o);
+    float t[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float ri = f4(R.a, i);
+      t[i] = f4(w, i) * (ri - kOmega * (ri - off[i]));
+    }
+    c0 += t[0] + t[1];
+    c1 += t[2] + t[3];
+    return 0.f;
+  }
+  float dot = 0.f, x[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float vi = f4(R.v, i), ri = f4(R.a, i);
+    const bool live = f4(R.s, i) != 0.f;
+    if (MODE == kUp) {
+      x[i] = live ? fmaf(kOmega, ri - (vi - off[i]), vi) : 0.f;
+      dot = fmaf(ri * x[i], wd, dot);
+    } else {
+      x[i] = live ? vi - off[i] : 0.f;
+      dot = fmaf(vi * x[i], wd, dot);
+    }
+  }
+  if (MODE == kUp) {
+    *reinterpret_cast<float4 *>(A.out + o) = make_float4(x[0], x[1], x[2], x[3]);
+  } else {
+    *reinterpret_cast<float4 *>(A.out + o) = R.v;
+    *reinterpret_cast<float4 *>(A.out2 + o) = make_float4(x[0], x[1], x[2], x[3]);
+  }
+  return dot;
+}
+
+// kDown: the level-1 residual and pre-smoothed correction of a lane's two
+// boxes in level-1 row `row`.
+__device__ __forceinline__ void coarse_out(const Mg0 &A, int64_t row, int X, float c0, float c1) {
+  if (X < A.nx1) {
+    A.out[row + X] = c0;
+    A.out2[row + X] = kOmega * c0 * __ldg(A.ia1 + row + X);
+  }
+  if (X + 1 < A.nx1) {
+    A.out[row + X + 1] = c1;
+    A.out2[row + X + 1] = kOmega * c1 * __ldg(A.ia1 + row + X + 1);
+  }
+}
+
+// What a lane keeps for all its rows: x-face weights, cell factors.
+struct Lane0 {
+  float hx[4], fL, fR, wd;
+  int kc, kcol;
+};
+__device__ __forceinline__ Lane0 lane0(const Mg0 &A, int xl, int y, int z, int kmin) {
+  Lane0 L;
+  const int mask = A.cg.B - 1, lg = A.cg.lgB;
+  const bool half = A.g.boundary == EIK_BOUNDARY_HALF_CELL;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    L.hx[i] = (half && (xl + i == 0 || xl + i == A.g.nx - 1)) ? 0.5f : 1.f;
+  const int row = A.cg.cx * ((y >> lg) + A.cg.cy * (z >> lg));
+  const int xc = min(xl, A.g.nx - 1);
+  L.kcol = xc >> lg;
+  L.kc = __ldg(A.kx + row + L.kcol);
+  L.fL = (xc > 0 && (xc & mask) == 0) ? p2f(L.kc - __ldg(A.kx + row + L.kcol - 1)) : 1.f;
+  L.fR = (xl + 4 < A.g.nx && ((xl + 4) & mask) == 0)
+             ? p2f(L.kc - __ldg(A.kx + row + L.kcol + 1)) : 1.f;
+  L.wd = p2f(2 * (kmin - L.kc));
+  return L;
+}
+
+// End of a pass with a dot product: <r, z> (kUp) or <p, q> (kDir).
+template <int MODE>
+__device__ void dot0_end(float dot, MgCtl *ctl, double *part) {
   __shared__ double sh[32];
   __shared__ int flag;
-  if (ctl->done) return;
-  const int kmin = ctl->kmin;
-  float rz = 0.f;
-  auto u = [&](int64_t j, int xj, int yj, int zj) {
-    return fmaf(w[j], L1.y[lin<DIM>(xj >> 1, yj >> 1, zj >> 1, L1.nx, L1.ny)], kOmega * r[j]);
-  };
-  MG_ROWS(g.ny, g.nz) MG_COLS(g.nx) {
-    const int64_t i = x + (int64_t)px * rr;
-    if (s32[i] == 0.f) {
-      zv[i] = 0.f;
-      continue;
-    }
-    const int ki = kx_at(cg, x, y, z, kx);
-    const float ui = u(i, x, y, z);
-    const float Au = ui - nb0<DIM>(g, cg, px, s32, kx, x, y, z, ki, u);
-    const float zi = fmaf(kOmega, r[i] - Au, ui);
-    zv[i] = zi;
-    rz = fmaf(r[i] * zi, wdot(ki, kmin), rz);
-  }
-  const double bs = block_sum((double)rz, sh);
-  if (threadIdx.x == 0) part[block_id()] = bs;
-  if (!last_block_2d(&ctl->counter[0], &flag)) return;
-  const double tot = sum_partials(part, block_count(), sh);
-  if (threadIdx.x == 0) {
+  const double bs = block_sum((double)dot, sh);
+  if (threadIdx.x == 0) part[blockIdx.x] = bs;
+  if (!last_block(&ctl->counter[MODE == kUp ? 0 : 1], &flag)) return;
+  const double tot = sum_partials(part, gridDim.x, sh);
+  if (threadIdx.x != 0) return;
+  if (MODE == kUp) {
     ctl->beta = ctl->first ? 0.0 : tot / ctl->rho;
     ctl->rho = tot;
     ctl->counter[0] = 0u;
@@ -536,40 +591,7 @@ k_mg_up0(Grid g, CellGrid cg, int px, const float *__restrict__ s32, const int *
       ctl->stalled = 1;
       ctl->done = 1;
     }
-  }
-}
-
-// p = z + beta p_old, q = A p, <p, q>; alpha = rho / <p, q>.
-template <int DIM>
-__global__ void __launch_bounds__(kThreads)
-k_mg_dir(Grid g, CellGrid cg, int px, const float *__restrict__ s32, const int *__restrict__ kx,
-         const float *__restrict__ zv, const float *__restrict__ p_old, float *__restrict__ p_new,
-         float *__restrict__ q, MgCtl *ctl, double *part) {
-  __shared__ double sh[32];
-  __shared__ int flag;
-  if (ctl->done) return;
-  const int kmin = ctl->kmin;
-  const float beta = (float)ctl->beta;
-  const bool first = ctl->first != 0;
-  float pq = 0.f;
-  auto pv = [&](int64_t j, int, int, int) { return first ? zv[j] : fmaf(beta, p_old[j], zv[j]); };
-  MG_ROWS(g.ny, g.nz) MG_COLS(g.nx) {
-    const int64_t i = x + (int64_t)px * rr;
-    const float pi = pv(i, x, y, z);
-    float qi = 0.f;
-    if (s32[i] != 0.f) {
-      const int ki = kx_at(cg, x, y, z, kx);
-      qi = pi - nb0<DIM>(g, cg, px, s32, kx, x, y, z, ki, pv);
-      pq = fmaf(pi * qi, wdot(ki, kmin), pq);
-    }
-    p_new[i] = pi;
-    q[i] = qi;
-  }
-  const double bs = block_sum((double)pq, sh);
-  if (threadIdx.x == 0) part[block_id()] = bs;
-  if (!last_block_2d(&ctl->counter[1], &flag)) return;
-  const double tot = sum_partials(part, block_count(), sh);
-  if (threadIdx.x == 0) {
+  } else {
     ctl->counter[1] = 0u;
     ctl->first = 0;
     if (!(tot > 0.0) || !isfinite(tot)) {
@@ -582,44 +604,292 @@ k_mg_dir(Grid g, CellGrid cg, int px, const float *__restrict__ s32, const int *
   }
 }
 
-// d += alpha p, r -= alpha q, and the stopping tests.
+constexpr int kRows2 = 8;       // 2D: rows per warp tile
+// 2D: every warp marches its tiles of 128 x kRows2 downwards.
+template <int MODE>
 __global__ void __launch_bounds__(kThreads)
-k_mg_step(Grid g, int px, const float *__restrict__ p, const float *__restrict__ q,
-          const float *__restrict__ xref, float *__restrict__ d, float *__restrict__ r, MgCtl *ctl,
-          double *part, int nblk_part) {
-  __shared__ double sh[32];
+k_mg0_2d(const Mg0 A, int tiles_x, int ntiles, MgCtl *ctl, double *part) {
+  if (ctl->done) return;
+  const int kmin = ctl->kmin, lane = threadIdx.x & 31;
+  const float beta = (float)ctl->beta;
+  const bool first = ctl->first != 0;
+  const int mask = A.cg.B - 1, lg = A.cg.lgB;
+  const bool half = A.g.boundary == EIK_BOUNDARY_HALF_CELL;
+  const int nw = gridDim.x * (blockDim.x >> 5);
+  float dot = 0.f;
+  for (int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < ntiles; t += nw) {
+    const int ty = t / tiles_x, x0 = (t - ty * tiles_x) * 128, y0 = ty * kRows2;
+    const int xl = x0 + 4 * lane;
+    const bool act = xl < A.px;
+    const Lane0 L = lane0(A, xl, y0, 0, kmin);
+    const int nrow = min(kRows2, A.g.ny - y0);
+    // the node left (lane 0) or right (lane 31) of the tile
+    const int xr = (lane == 0) ? x0 - 1 : x0 + 128;
+    const bool rim = (lane == 0 && x0 > 0) || (lane == 31 && x0 + 128 < A.g.nx);
+    const int X = xl >> 1;
+    auto parents = [&](int y, float &a, float &b, float &c) {
+      a = b = c = 0.f;
+      if (MODE != kUp || y < 0 || y >= A.g.ny) return;
+      const float *q = A.y1 + (int64_t)(y >> 1) * A.nx1;
+      if (X < A.nx1) a = __ldg(q + X);
+      if (X + 1 < A.nx1) b = __ldg(q + X + 1);
+      if (rim) c = __ldg(q + (xr >> 1));
+    };
+    auto load = [&](int y, Row0 &R, float &ur) {
+      float a, b, c;
+      parents(y, a, b, c);
+      const bool in = y >= 0 && y < A.g.ny;
+      R = row0_load<MODE>(A, (int64_t)y * A.px + xl, in && act, a, b, beta, first);
+      ur = rim0<MODE>(A, (int64_t)y * A.px + xr, in && rim, c, beta, first);
+    };
+    Row0 C, N;
+    float urc, urn;
+    load(y0 - 1, C, urc);
+    float4 um = mul4f(C.s, C.v);
+    load(y0, C, urc);
+    float4 uc = mul4f(C.s, C.v);
+    float c0 = 0.f, c1 = 0.f;
+#pragma unroll 2
+    for (int j = 0; j < nrow; ++j) {
+      const int y = y0 + j;
+      load(y + 1, N, urn);
+      const float4 un = mul4f(N.s, N.v);
+      float fU = 1.f, fD = 1.f;
+      if ((y & mask) == 0 && y > 0)
+        fU = p2f(L.kc - __ldg(A.kx + A.cg.cx * ((y >> lg) - 1) + L.kcol));
+      if (((y + 1) & mask) == 0 && y + 1 < A.g.ny)
+        fD = p2f(L.kc - __ldg(A.kx + A.cg.cx * ((y >> lg) + 1) + L.kcol));
+      const float hy = (half && (y == 0 || y == A.g.ny - 1)) ? 0.5f : 1.f;
+      float uL = __shfl_up_sync(0xffffffffu, uc.w, 1);
+      float uR = __shfl_down_sync(0xffffffffu, uc.x, 1);
+      if (lane == 0) uL = urc;
+      if (lane == 31) uR = urc;
+      const float xs[4] = {fmaf(uL, L.fL, uc.y), uc.x + uc.z, uc.y + uc.w, fmaf(uR, L.fR, uc.z)};
+      float off[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        off[i] = f4(C.s, i) * fmaf(hy, xs[i], L.hx[i] * fmaf(f4(um, i), fU, f4(un, i) * fD));
+      if (act) dot += row0_out<MODE>(A, (int64_t)y * A.px + xl, C, off, L.wd, c0, c1);
+      if (MODE == kDown && ((j & 1) || j == nrow - 1)) {
+        coarse_out(A, (int64_t)(y >> 1) * A.nx1, X, c0, c1);
+        c0 = c1 = 0.f;
+      }
+      um = uc;
+      uc = un;
+      C = N;
+      urc = urn;
+    }
+  }
+  if (MODE != kDown) dot0_end<MODE>(dot, ctl, part);
+}
+
+constexpr int kRows3 = 16;                  // 3D: rows per block tile
+constexpr int kThreads3 = 32 * (kRows3 / 2 + 1);
+// 3D: a block marches its tile of 128 x kRows3 columns through zc planes
+// (even).  Warp w < 8 owns rows y0 + 2 w and the next; warp 8 supplies u of the
+// rows y0 - 1 and y0 + 16.  Shared memory holds three planes of u (the one
+// being written, the one in use, and the one that slower warps may still
+// read), so a plane takes one barrier.
+template <int MODE>
+__global__ void __launch_bounds__(kThreads3, 2)
+k_mg0_3d(const Mg0 A, int tiles_x, int tiles_y, int zc, int ntiles, MgCtl *ctl, double *part) {
+  __shared__ float4 us[3][kRows3 + 2][32];
+  if (ctl->done) return;
+  const int kmin = ctl->kmin, lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
+  const float beta = (float)ctl->beta;
+  const bool first = ctl->first != 0;
+  const int mask = A.cg.B - 1, lg = A.cg.lgB;
+  const bool half = A.g.boundary == EIK_BOUNDARY_HALF_CELL;
+  const bool rows = wi < kRows3 / 2;
+  float dot = 0.f;
+  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    const int tz = t / (tiles_x * tiles_y), rem = t - tz * tiles_x * tiles_y;
+    const int ty = rem / tiles_x, x0 = (rem - ty * tiles_x) * 128;
+    const int y0 = ty * kRows3, z0 = tz * zc;
+    const int nz = min(zc, A.g.nz - z0);
+    const int xl = x0 + 4 * lane;
+    const bool act = xl < A.px;
+    const int xr = (lane == 0) ? x0 - 1 : x0 + 128;
+    const bool rim = rows && ((lane == 0 && x0 > 0) || (lane == 31 && x0 + 128 < A.g.nx));
+    const int X = xl >> 1;
+    // the warp's two rows and their places in shared memory
+    const int yr[2] = {rows ? y0 + 2 * wi : y0 - 1, rows ? y0 + 2 * wi + 1 : y0 + kRows3};
+    const int pr[2] = {rows ? 1 + 2 * wi : 0, rows ? 2 + 2 * wi : kRows3 + 1};
+    const Lane0 L = lane0(A, xl, min(max(yr[0], 0), A.g.ny - 1), z0, kmin);
+    const int layer = A.cg.cx * A.cg.cy;
+    const int crow = L.kcol + A.cg.cx * (min(max(yr[0], 0), A.g.ny - 1) >> lg) + layer * (z0 >> lg);
+    float fU = 1.f, fD = 1.f;
+    if (rows && yr[0] > 0 && yr[0] < A.g.ny && (yr[0] & mask) == 0)
+      fU = p2f(L.kc - __ldg(A.kx + crow - A.cg.cx));
+    if (rows && yr[1] + 1 < A.g.ny && ((yr[1] + 1) & mask) == 0)
+      fD = p2f(L.kc - __ldg(A.kx + crow + A.cg.cx));
+    float hy[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) hy[e] = (half && (yr[e] == 0 || yr[e] == A.g.ny - 1)) ? 0.5f : 1.f;
+    auto load = [&](int z, Row0 (&R)[2], float (&ur)[2]) {
+      const bool inz = z >= 0 && z < A.g.nz;
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const bool in = inz && yr[e] >= 0 && yr[e] < A.g.ny;
+        float a = 0.f, b = 0.f, c = 0.f;
+        if (MODE == kUp && in) {
+          const float *q = A.y1 + (int64_t)A.nx1 * ((yr[e] >> 1) + (int64_t)A.ny1 * (z >> 1));
+          if (X < A.nx1) a = __ldg(q + X);
+          if (X + 1 < A.nx1) b = __ldg(q + X + 1);
+          if (rim) c = __ldg(q + (xr >> 1));
+        }
+        const int64_t o = (int64_t)A.px * (yr[e] + (int64_t)A.g.ny * z);
+        R[e] = row0_load<MODE>(A, o + xl, in && act, a, b, beta, first);
+        ur[e] = rim0<MODE>(A, o + xr, in && rim, c, beta, first);
+      }
+    };
+    Row0 C[2], N[2];
+    float urc[2], urn[2];
+    float4 um[2], uc[2];
+    load(z0 - 1, C, urc);
+#pragma unroll
+    for (int e = 0; e < 2; ++e) um[e] = mul4f(C[e].s, C[e].v);
+    load(z0, C, urc);
+    __syncthreads();   // the previous tile's planes are no longer read
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      uc[e] = mul4f(C[e].s, C[e].v);
+      us[0][pr[e]][lane] = uc[e];
+    }
+    float c0 = 0.f, c1 = 0.f;
+    int cur = 0;
+    for (int j = 0; j < nz; ++j) {
+      const int z = z0 + j;
+      load(z + 1, N, urn);
+      const int nxt = (cur == 2) ? 0 : cur + 1;
+      float4 un[2];
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        un[e] = mul4f(N[e].s, N[e].v);
+        us[nxt][pr[e]][lane] = un[e];
+      }
+      __syncthreads();
+      if (rows) {
+        float fP = 1.f, fN = 1.f;
+        if ((z & mask) == 0 && z > 0) fP = p2f(L.kc - __ldg(A.kx + crow - layer));
+        if (((z + 1) & mask) == 0 && z + 1 < A.g.nz) fN = p2f(L.kc - __ldg(A.kx + crow + layer));
+        const float hz = (half && (z == 0 || z == A.g.nz - 1)) ? 0.5f : 1.f;
+        const float4 yu = us[cur][pr[0] - 1][lane], yd = us[cur][pr[1] + 1][lane];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          float uL = __shfl_up_sync(0xffffffffu, uc[e].w, 1);
+          float uR = __shfl_down_sync(0xffffffffu, uc[e].x, 1);
+          if (lane == 0) uL = urc[e];
+          if (lane == 31) uR = urc[e];
+          const float4 up = (e == 0) ? yu : uc[0], dn = (e == 0) ? uc[1] : yd;
+          const float gu = (e == 0) ? fU : 1.f, gd = (e == 0) ? 1.f : fD;
+          const float xs[4] = {fmaf(uL, L.fL, uc[e].y), uc[e].x + uc[e].z, uc[e].y + uc[e].w,
+                               fmaf(uR, L.fR, uc[e].z)};
+          const float wx = hy[e] * hz;
+          float off[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float ys = fmaf(f4(up, i), gu, f4(dn, i) * gd);
+            const float zs = fmaf(f4(um[e], i), fP, f4(un[e], i) * fN);
+            off[i] = f4(C[e].s, i) * fmaf(wx, xs[i], L.hx[i] * fmaf(hz, ys, hy[e] * zs));
+          }
+          if (act && yr[e] < A.g.ny) {
+            const int64_t o = (int64_t)A.px * (yr[e] + (int64_t)A.g.ny * z) + xl;
+            dot += row0_out<MODE>(A, o, C[e], off, L.wd, c0, c1);
+          }
+        }
+        if (MODE == kDown && ((j & 1) || j == nz - 1)) {
+          if (yr[0] < A.g.ny)
+            coarse_out(A, (int64_t)A.nx1 * ((yr[0] >> 1) + (int64_t)A.ny1 * (z >> 1)), X, c0, c1);
+          c0 = c1 = 0.f;
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        um[e] = uc[e];
+        uc[e] = un[e];
+        C[e] = N[e];
+        urc[e] = urn[e];
+      }
+      cur = nxt;
+    }
+  }
+  if (MODE != kDown) dot0_end<MODE>(dot, ctl, part);
+}
+
+// Largest of the threads' values, in all threads of warp 0.
+__device__ __forceinline__ unsigned block_max_bits(unsigned v, unsigned *sh) {
+  v = __reduce_max_sync(0xffffffffu, v);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    v = (threadIdx.x < (blockDim.x >> 5)) ? sh[threadIdx.x] : 0u;
+    v = __reduce_max_sync(0xffffffffu, v);
+  }
+  return v;
+}
+
+// d += alpha p, r -= alpha q, and the stopping tests; n4 float4 groups of the
+// pitched arrays (their padding columns are zero and stay so).
+__global__ void __launch_bounds__(kThreads)
+k_mg_step(int64_t n4, const float4 *__restrict__ p, const float4 *__restrict__ q,
+          const float4 *__restrict__ xref, float4 *__restrict__ d, float4 *__restrict__ r,
+          MgCtl *ctl, double *part) {
+  __shared__ unsigned sh[32];
   __shared__ int flag;
   if (ctl->done) return;
   const float alpha = (float)ctl->alpha;
   const int mode = ctl->mode;
   const float theta = ctl->theta;
   float rmax = 0.f, viol = 0.f;
-  for (int rr = blockIdx.y; rr < g.ny * g.nz; rr += gridDim.y) MG_COLS(g.nx) {
-    const int64_t i = x + (int64_t)px * rr;
-    const float di = fmaf(alpha, p[i], d[i]);
-    const float ri = fmaf(-alpha, q[i], r[i]);
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const float4 pi = p[i], qi = q[i];
+    float4 di = d[i], ri = r[i];
+    di = make_float4(fmaf(alpha, pi.x, di.x), fmaf(alpha, pi.y, di.y), fmaf(alpha, pi.z, di.z),
+                     fmaf(alpha, pi.w, di.w));
+    ri = make_float4(fmaf(-alpha, qi.x, ri.x), fmaf(-alpha, qi.y, ri.y), fmaf(-alpha, qi.z, ri.z),
+                     fmaf(-alpha, qi.w, ri.w));
     d[i] = di;
     r[i] = ri;
-    rmax = fmaxf(rmax, fabsf(ri));
-    if (mode == 1 && fabsf(ri) > theta * fabsf(xref[i] + di)) viol = 1.f;
+    rmax = fmaxf(rmax, fmaxf(fmaxf(fabsf(ri.x), fabsf(ri.y)), fmaxf(fabsf(ri.z), fabsf(ri.w))));
+    if (mode == 1) {
+      const float4 xi = __ldg(xref + i);
+      if (fabsf(ri.x) > theta * fabsf(xi.x + di.x) || fabsf(ri.y) > theta * fabsf(xi.y + di.y) ||
+          fabsf(ri.z) > theta * fabsf(xi.z + di.z) || fabsf(ri.w) > theta * fabsf(xi.w + di.w))
+        viol = 1.f;
+    }
   }
-  const double b1 = block_max((double)rmax, sh);
-  const double b2 = block_max((double)viol, sh);
+  // (maxima of non-negative floats are maxima of their bits: the integer
+  // reductions keep this off the FP64 pipe)
+  const unsigned b1 = block_max_bits(__float_as_uint(rmax), sh);
+  const unsigned b2 = (unsigned)__syncthreads_or(viol != 0.f);
+  unsigned *ip = reinterpret_cast<unsigned *>(part);
   if (threadIdx.x == 0) {
-    part[block_id()] = b1;
-    part[nblk_part + block_id()] = b2;
+    ip[2 * blockIdx.x] = b1;
+    ip[2 * blockIdx.x + 1] = b2;
   }
-  if (!last_block_2d(&ctl->counter[2], &flag)) return;
-  const double rm = max_partials(part, block_count(), sh);
-  const double vi = max_partials(part + nblk_part, block_count(), sh);
+  if (!last_block(&ctl->counter[2], &flag)) return;
+  unsigned m1 = 0, m2 = 0;
+  for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
+    const uint2 v = __ldcg(reinterpret_cast<const uint2 *>(ip) + b);
+    m1 = max(m1, v.x);
+    m2 |= v.y;
+  }
+  const float rm = __uint_as_float(block_max_bits(m1, sh));
+  const int vi = __syncthreads_or(m2 != 0u);
   if (threadIdx.x == 0) {
     ctl->counter[2] = 0u;
     ctl->iter += 1;
-    const bool conv = (mode == 0) ? (rm <= (double)ctl->thresh) : (vi == 0.0);
+    const bool conv = (mode == 0) ? (rm <= ctl->thresh) : (vi == 0);
     if (!isfinite(rm)) {
       ctl->status = EIK_ERR_BREAKDOWN;
       ctl->done = 1;
     } else if (conv || ctl->iter >= ctl->max_iter) {
+      ctl->done = 1;
+    } else if (rm > ctl->r_limit) {
+      ctl->stalled = 2;
       ctl->done = 1;
     }
   }
@@ -678,7 +948,7 @@ void mg_destroy(MgState *mg) {
     if (e) cudaEventDestroy(e);
   for (size_t l = 1; l < mg->lv.size(); ++l) {
     MgLevel &L = mg->lv[l];
-    void *arr[] = {L.a, L.ia, L.c, L.k, L.g, L.y};
+    void *arr[] = {L.a, L.ia, L.c, L.k, L.g, L.yp, L.y};
     for (void *p : arr)
       if (p) cudaFree(p);
   }
@@ -716,7 +986,7 @@ eik_status mg_create(MgState **out, const Grid &g, const CellGrid &cg, int px, i
     ok = cudaMalloc(&L.a, 4 * m) == cudaSuccess && cudaMalloc(&L.ia, 4 * m) == cudaSuccess &&
          cudaMalloc(&L.c, 4 * kDirs * m) == cudaSuccess &&
          cudaMalloc(&L.k, 4 * m) == cudaSuccess && cudaMalloc(&L.g, 4 * m) == cudaSuccess &&
-         cudaMalloc(&L.y, 4 * m) == cudaSuccess;
+         cudaMalloc(&L.yp, 4 * m) == cudaSuccess && cudaMalloc(&L.y, 4 * m) == cudaSuccess;
     mg->lv.push_back(L);
   }
   const size_t np = (size_t)g.ny * g.nz * px;
@@ -743,27 +1013,34 @@ eik_status mg_create(MgState **out, const Grid &g, const CellGrid &cg, int px, i
   return EIK_OK;
 }
 
-// Row-strided launch grid of a level: columns by blockIdx.x, rows by
-// blockIdx.y, at most cap blocks.
-static dim3 grid2(const MgState *mg, int nx, int64_t rows) {
-  const int gx = std::max(1, std::min((nx + kThreads - 1) / kThreads, mg->cap));
+// Row-strided launch shape of a level: blocks of kThreads threads, as many
+// columns as the row has up to kThreads (a power of two), rows beside each
+// other; at most cap blocks.
+struct Shape {
+  dim3 grid, block;
+};
+static Shape shape_of(const MgState *mg, const MgLevel &L) {
+  int bx = 1;
+  while (bx < L.nx && bx < kThreads) bx *= 2;
+  const int by = kThreads / bx;
+  const int gx = std::max(1, std::min((L.nx + bx - 1) / bx, mg->cap));
+  const int64_t rows = ((int64_t)L.ny * L.nz + by - 1) / by;
   const int gy = (int)std::max<int64_t>(1, std::min<int64_t>(rows, mg->cap / gx));
-  return dim3((unsigned)gx, (unsigned)gy, 1);
-}
-static dim3 grid_of(const MgState *mg, const MgLevel &L) {
-  return grid2(mg, L.nx, (int64_t)L.ny * L.nz);
+  return Shape{dim3((unsigned)gx, (unsigned)gy, 1), dim3((unsigned)bx, (unsigned)by, 1)};
 }
 
 eik_status mg_setup(MgState *mg, const MgFine &f, int kmin, cudaStream_t s) {
   const Grid &g = mg->g;
-  k_mg_weights<<<grid_of(mg, mg->lv[0]), kThreads, 0, s>>>(g, mg->cg, mg->px, f.s32, f.kx, f.St,
-                                                            mg->w);
+  const Shape s0 = shape_of(mg, mg->lv[0]);
+  k_mg_weights<<<s0.grid, s0.block, 0, s>>>(g, mg->cg, mg->px, f.s32, f.kx, f.St, mg->w);
   MgLevel &L1 = mg->lv[1];
-  k_mg_coarsen0<<<grid_of(mg, L1), kThreads, 0, s>>>(g, mg->cg, mg->px, f.s32, f.kx, mg->w, L1);
+  const Shape s1 = shape_of(mg, L1);
+  k_mg_coarsen0<<<s1.grid, s1.block, 0, s>>>(g, mg->cg, mg->px, f.s32, f.kx, mg->w, L1);
   mg->launches += 2;
   for (size_t l = 1; l + 1 < mg->lv.size(); ++l) {
     MgLevel &C = mg->lv[l + 1];
-    k_mg_coarsen<<<grid_of(mg, C), kThreads, 0, s>>>(mg->lv[l], C);
+    const Shape sh = shape_of(mg, C);
+    k_mg_coarsen<<<sh.grid, sh.block, 0, s>>>(mg->lv[l], C);
     mg->launches++;
   }
   GCK(cudaGetLastError());
@@ -782,31 +1059,72 @@ static int tail_start(const MgState *mg) {
   return l;
 }
 
+// One level-0 pass.
+template <int MODE>
+static void launch0(MgState *mg, const MgFine &f, int set, cudaStream_t s) {
+  const Grid &g = mg->g;
+  Mg0 a{};
+  a.g = g;
+  a.cg = mg->cg;
+  a.px = mg->px;
+  a.s32 = f.s32;
+  a.kx = f.kx;
+  a.w = mg->w;
+  a.r = f.r;
+  a.z = mg->z;
+  a.p_old = mg->p[set];
+  a.out = (MODE == kDown) ? mg->lv[1].g : (MODE == kUp) ? mg->z : mg->p[1 - set];
+  a.out2 = (MODE == kDown) ? mg->lv[1].yp : mg->q;
+  a.ia1 = mg->lv[1].ia;
+  a.y1 = mg->lv[1].y;
+  a.nx1 = mg->lv[1].nx;
+  a.ny1 = mg->lv[1].ny;
+  const int tx = (g.nx + 127) / 128;
+  if (g.ndim == 2) {
+    const int64_t nt = (int64_t)tx * ((g.ny + kRows2 - 1) / kRows2);
+    const int64_t nb = (nt + kThreads / 32 - 1) / (kThreads / 32);
+    k_mg0_2d<MODE><<<(int)std::min<int64_t>(nb, mg->cap), kThreads, 0, s>>>(a, tx, (int)nt,
+                                                                            mg->ctl, mg->part);
+  } else {
+    // planes per tile: as many as leave two blocks per SM (each tile reads
+    // two planes beside its own); divisors of the cell edge
+    const int ty = (g.ny + kRows3 - 1) / kRows3;
+    int zc = 16;
+    while (zc > 2 && (int64_t)tx * ty * ((g.nz + zc - 1) / zc) < mg->cap / 4) zc /= 2;
+    const int64_t nt = (int64_t)tx * ty * ((g.nz + zc - 1) / zc);
+    k_mg0_3d<MODE><<<(int)std::min<int64_t>(nt, mg->cap), kThreads3, 0, s>>>(
+        a, tx, ty, zc, (int)nt, mg->ctl, mg->part);
+  }
+}
+
 template <int DIM>
 static void launch_iter_d(MgState *mg, const MgFine &f, int set, cudaStream_t s) {
   const Grid &g = mg->g;
   const int L = (int)mg->lv.size() - 1;   // coarsest level index
-  const dim3 g0 = grid_of(mg, mg->lv[0]);
-  k_mg_down0<DIM><<<grid_of(mg, mg->lv[1]), kThreads, 0, s>>>(
-      g, mg->cg, mg->px, f.s32, f.kx, mg->w, f.r, mg->lv[1], mg->ctl);
+  launch0<kDown>(mg, f, set, s);
   // levels 1 .. ts - 1 one launch each way; ts .. L in the single-block tail
   const int ts = tail_start(mg);
-  for (int l = 1; l < ts; ++l)
-    k_mg_down<DIM><<<grid_of(mg, mg->lv[l + 1]), kThreads, 0, s>>>(mg->lv[l], mg->lv[l + 1],
-                                                                     mg->ctl);
+  for (int l = 1; l < ts; ++l) {
+    const Shape sh = shape_of(mg, mg->lv[l + 1]);
+    k_mg_down<DIM><<<sh.grid, sh.block, 0, s>>>(mg->lv[l], mg->lv[l + 1], mg->ctl);
+  }
   MgTail T{};
   for (int l = ts; l <= L; ++l) T.lv[l] = mg->lv[l];
   T.s = ts;
   T.L = L;
   k_mg_tail<DIM><<<1, kTailThreads, 0, s>>>(T, mg->ctl);
-  for (int l = ts - 1; l >= 1; --l)
-    k_mg_up<DIM><<<grid_of(mg, mg->lv[l]), kThreads, 0, s>>>(mg->lv[l], mg->lv[l + 1], mg->ctl);
-  k_mg_up0<DIM><<<g0, kThreads, 0, s>>>(g, mg->cg, mg->px, f.s32, f.kx, mg->w, f.r, mg->lv[1], mg->z,
-                                   mg->ctl, mg->part);
-  k_mg_dir<DIM><<<g0, kThreads, 0, s>>>(g, mg->cg, mg->px, f.s32, f.kx, mg->z, mg->p[set],
-                                   mg->p[1 - set], mg->q, mg->ctl, mg->part);
-  k_mg_step<<<g0, kThreads, 0, s>>>(g, mg->px, mg->p[1 - set], mg->q, f.xref, f.d, f.r, mg->ctl,
-                                    mg->part, mg->cap);
+  for (int l = ts - 1; l >= 1; --l) {
+    const Shape sh = shape_of(mg, mg->lv[l]);
+    k_mg_up<DIM><<<sh.grid, sh.block, 0, s>>>(mg->lv[l], mg->lv[l + 1], mg->ctl);
+  }
+  launch0<kUp>(mg, f, set, s);
+  launch0<kDir>(mg, f, set, s);
+  const int64_t n4 = (int64_t)(mg->px / 4) * g.ny * g.nz;
+  const int nb = (int)std::max<int64_t>(1, std::min<int64_t>((n4 + kThreads - 1) / kThreads, mg->cap));
+  auto v4 = [](const float *p) { return reinterpret_cast<const float4 *>(p); };
+  k_mg_step<<<nb, kThreads, 0, s>>>(n4, v4(mg->p[1 - set]), v4(mg->q), v4(f.xref),
+                                    reinterpret_cast<float4 *>(f.d),
+                                    reinterpret_cast<float4 *>(f.r), mg->ctl, mg->part);
 }
 
 // One PCG iteration with the kernels specialised to the grid's dimension.
@@ -840,6 +1158,7 @@ eik_status mg_inner(MgState *mg, const MgFine &f, MixCtl *h_st, cudaStream_t s) 
   c.mode = h_st->mode;
   c.thresh = h_st->thresh;
   c.theta = h_st->theta;
+  c.r_limit = kMaxGrowth * (float)h_st->r_inf;
   c.first = 1;
   *mg->h_ctl = c;
   GCK(cudaMemcpyAsync(mg->ctl, mg->h_ctl, sizeof(MgCtl), cudaMemcpyHostToDevice, s));

@@ -740,6 +740,9 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
   int total = *total_io, outer = 0;
   double best_cw = INFINITY, last_cw = INFINITY;
   int stall = 0;
+  // set once an inner solve has come apart: the later ones aim at the smaller
+  // reduction of the first step, which they reach before they do
+  bool careful = false;
   eik_status result = EIK_ERR_NOT_CONVERGED;
   for (;;) {
     MixCtl init{};
@@ -773,7 +776,7 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
     // progress is then judged only once it is finite)
     // a step that recovers from a bad correction (an inner solve that lost
     // conjugacy late) counts as progress too
-    const bool recovering = cw < 0.1 * last_cw;
+    const bool recovering = cw < 0.5 * last_cw;
     last_cw = cw;
     if (!std::isfinite(cw) || cw < 0.5 * best_cw) {
       if (std::isfinite(cw)) best_cw = cw;
@@ -803,7 +806,7 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
     st.fault = 0;
     st.max_iter = std::max(1, a.opt.max_iter - total);
     st.withhold = (a.opt.test_flags & 1) ? 1 : 0;
-    st.mode = (outer == 0 || !std::isfinite(cw)) ? 0 : 1;
+    st.mode = (outer == 0 || !std::isfinite(cw) || careful) ? 0 : 1;
     st.thresh = (float)(red * st.r_inf);
     st.theta = (float)std::max(0.5 * tol, 1e-3 * cw);
     if (m->batch) {
@@ -906,6 +909,10 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
       g_msg = "inner CG breakdown";
       result = EIK_ERR_BREAKDOWN;
       break;
+    }
+    if (m->h_st->stalled == 2 && !careful) {
+      careful = true;   // the correction is dropped
+      continue;
     }
     k_mixed_update<<<blocks(g.n), kThreads, 0, s>>>(g.n, g.nx, m->px, m->d32, m->x64);
     m->launches[5]++;
