@@ -422,7 +422,7 @@ __global__ void __launch_bounds__(kTailThreads) k_mg_tail(MgTail T, const MgCtl 
 // (z in 3D, y in 2D), a shuffle (x) and shared memory (y in 3D); gathering
 // them per node, as these passes did before, formed every u five or seven
 // times from up to four loads each and left them bound by load latency
-// (256^3: 1.19 ms an iteration for the three, 0.42 ms now; 2048^2: 163 us, 83 us).
+// (256^3: 1.19 ms an iteration for the three, 0.23 ms now; 2048^2: 163 us, 83 us).
 //   down (kDown): v = r;                g1 = sum over the box of w (r - omega (r - A' v)),
 //   up   (kUp):   v = omega r + w y1,   z = v + omega (r - A v), <r, z>,
 //   dir  (kDir):  v = z + beta p_old,   p = v, q = A v, <p, q>.
@@ -453,7 +453,7 @@ __device__ __forceinline__ float f4(const float4 &v, int i) {
 }
 
 // One row of a tile at pitched offset o: sigma, v and the arrays that the
-// output needs later (a: r in kDown and kUp).  y1x/y1y: the parents'
+// output needs later (a: r in kDown and kUp, w: in kDown).  y1x/y1y: the parents'
 // corrections of the lane's two column pairs.
 struct Row0 {
   float4 s, v, a, w;
@@ -468,6 +468,7 @@ __device__ __forceinline__ Row0 row0_load(const Mg0 &A, int64_t o, bool in, floa
   R.s = ld4g(A.s32 + o);
   if (MODE == kDown) {
     R.a = R.v = ld4g(A.r + o);
+    R.w = ld4g(A.w + o);
   } else if (MODE == kUp) {
     R.a = ld4g(A.r + o);
     const float4 w = ld4g(A.w + o);
@@ -504,12 +505,11 @@ template <int MODE>
 __device__ __forceinline__ float row0_out(const Mg0 &A, int64_t o, const Row0 &R,
                                           const float (&off)[4], float wd, float &c0, float &c1) {
   if (MODE == kDown) {
-    const float4 w = ld4g(A.w + o);
     float t[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const float ri = f4(R.a, i);
-      t[i] = f4(w, i) * (ri - kOmega * (ri - off[i]));
+      t[i] = f4(R.w, i) * (ri - kOmega * (ri - off[i]));
     }
     c0 += t[0] + t[1];
     c1 += t[2] + t[3];
@@ -684,23 +684,47 @@ k_mg0_2d(const Mg0 A, int tiles_x, int ntiles, MgCtl *ctl, double *part) {
 }
 
 constexpr int kRows3 = 16;                  // 3D: rows per block tile
-constexpr int kThreads3 = 32 * (kRows3 / 2 + 1);
+constexpr int kThreads3 = 32 * (kRows3 / 2);
+constexpr int kStages3 = 3;                 // planes of input in flight or in use
+constexpr int kPlane3 = (kRows3 + 2) * 32;  // float4 of one array and plane
+constexpr size_t kSmem3 = sizeof(float4) * kPlane3 * (3 * kStages3 + 3);
+
+// 16 bytes of global memory into shared memory, zeros where !in.
+__device__ __forceinline__ void copy16(float4 *dst, const float *src, bool in) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                   (unsigned)__cvta_generic_to_shared(dst)),
+               "l"(src), "r"(in ? 16 : 0)
+               : "memory");
+}
+
 // 3D: a block marches its tile of 128 x kRows3 columns through zc planes
-// (even).  Warp w < 8 owns rows y0 + 2 w and the next; warp 8 supplies u of the
-// rows y0 - 1 and y0 + 16.  Shared memory holds three planes of u (the one
-// being written, the one in use, and the one that slower warps may still
-// read), so a plane takes one barrier.
+// (even).  Warp w owns rows y0 + 2 w and the next; the first and the last warp
+// also supply u of the rows y0 - 1 and y0 + 16 (a ninth warp for them would cost
+// every thread 32 registers).  Every thread copies its own four columns of the
+// three input arrays into shared memory kStages3 - 1 planes ahead and reads
+// them back itself, so the copies need no barrier and no registers (the loads
+// of one plane ahead, in registers, left a block waiting for memory at every
+// plane: 0.42 ms for the three passes on 256^3, 0.23 ms this way).  Three planes of u are shared (the one being written, the one in
+// use, and the one that slower warps may still read), so a plane takes one
+// barrier.
 template <int MODE>
 __global__ void __launch_bounds__(kThreads3, 2)
 k_mg0_3d(const Mg0 A, int tiles_x, int tiles_y, int zc, int ntiles, MgCtl *ctl, double *part) {
-  __shared__ float4 us[3][kRows3 + 2][32];
+  extern __shared__ float4 sm3[];
+  float4 *us = sm3 + 3 * kStages3 * kPlane3;   // [3][kRows3 + 2][32]
   if (ctl->done) return;
   const int kmin = ctl->kmin, lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
   const float beta = (float)ctl->beta;
   const bool first = ctl->first != 0;
   const int mask = A.cg.B - 1, lg = A.cg.lgB;
   const bool half = A.g.boundary == EIK_BOUNDARY_HALF_CELL;
-  const bool rows = wi < kRows3 / 2;
+  const bool edge = wi == 0 || wi == kRows3 / 2 - 1;   // supplies a halo row
+  // the input arrays: sigma, and r, w (down, up) or z, p_old (dir)
+  const float *in1 = (MODE == kDir) ? A.z : A.r;
+  const float *in2 = (MODE == kDir) ? A.p_old : A.w;
+  // the warp's two rows in shared memory
+  const int pr[2] = {(1 + 2 * wi) * 32 + lane, (2 + 2 * wi) * 32 + lane};
+  const int ph = (wi == 0 ? 0 : kRows3 + 1) * 32 + lane;
   float dot = 0.f;
   for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const int tz = t / (tiles_x * tiles_y), rem = t - tz * tiles_x * tiles_y;
@@ -710,71 +734,156 @@ k_mg0_3d(const Mg0 A, int tiles_x, int tiles_y, int zc, int ntiles, MgCtl *ctl, 
     const int xl = x0 + 4 * lane;
     const bool act = xl < A.px;
     const int xr = (lane == 0) ? x0 - 1 : x0 + 128;
-    const bool rim = rows && ((lane == 0 && x0 > 0) || (lane == 31 && x0 + 128 < A.g.nx));
+    const bool rim = ((lane == 0 && x0 > 0) || (lane == 31 && x0 + 128 < A.g.nx));
     const int X = xl >> 1;
-    // the warp's two rows and their places in shared memory
-    const int yr[2] = {rows ? y0 + 2 * wi : y0 - 1, rows ? y0 + 2 * wi + 1 : y0 + kRows3};
-    const int pr[2] = {rows ? 1 + 2 * wi : 0, rows ? 2 + 2 * wi : kRows3 + 1};
-    const Lane0 L = lane0(A, xl, min(max(yr[0], 0), A.g.ny - 1), z0, kmin);
+    const int yr[2] = {y0 + 2 * wi, y0 + 2 * wi + 1};
+    const bool yin[2] = {yr[0] < A.g.ny, yr[1] < A.g.ny};
+    const int yh = (wi == 0) ? y0 - 1 : y0 + kRows3;
+    const bool hin = edge && yh >= 0 && yh < A.g.ny;
+    const Lane0 L = lane0(A, xl, min(yr[0], A.g.ny - 1), z0, kmin);
     const int layer = A.cg.cx * A.cg.cy;
-    const int crow = L.kcol + A.cg.cx * (min(max(yr[0], 0), A.g.ny - 1) >> lg) + layer * (z0 >> lg);
+    const int crow = L.kcol + A.cg.cx * (min(yr[0], A.g.ny - 1) >> lg) + layer * (z0 >> lg);
     float fU = 1.f, fD = 1.f;
-    if (rows && yr[0] > 0 && yr[0] < A.g.ny && (yr[0] & mask) == 0)
+    if (yr[0] > 0 && yr[0] < A.g.ny && (yr[0] & mask) == 0)
       fU = p2f(L.kc - __ldg(A.kx + crow - A.cg.cx));
-    if (rows && yr[1] + 1 < A.g.ny && ((yr[1] + 1) & mask) == 0)
+    if (yr[1] + 1 < A.g.ny && ((yr[1] + 1) & mask) == 0)
       fD = p2f(L.kc - __ldg(A.kx + crow + A.cg.cx));
     float hy[2];
 #pragma unroll
     for (int e = 0; e < 2; ++e) hy[e] = (half && (yr[e] == 0 || yr[e] == A.g.ny - 1)) ? 0.5f : 1.f;
-    auto load = [&](int z, Row0 (&R)[2], float (&ur)[2]) {
-      const bool inz = z >= 0 && z < A.g.nz;
+    // plane q of the march is z0 - 1 + q, q = 0 .. nz + 1
+    auto issue = [&](int q) {
+      const int z = z0 - 1 + q;
+      float4 *dst = sm3 + (q % kStages3) * 3 * kPlane3;
+      const bool inz = q < nz + 2 && z >= 0 && z < A.g.nz && act;
+      auto row = [&](int y, bool iny, int at) {
+        const bool in = inz && iny;
+        const int64_t o = in ? (int64_t)A.px * (y + (int64_t)A.g.ny * z) + xl : 0;
+        copy16(dst + at, A.s32 + o, in);
+        copy16(dst + kPlane3 + at, in1 + o, in);
+        copy16(dst + 2 * kPlane3 + at, in2 + o, in);
+      };
+#pragma unroll
+      for (int e = 0; e < 2; ++e) row(yr[e], yin[e], pr[e]);
+      if (edge) row(yh, hin, ph);
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    // what a plane needs beside them: the rim node's values, the parents'
+    // corrections (loaded a plane ahead)
+    struct Side {
+      float s[2], a[2], b[2], y0, y1, yc, yh0, yh1;   // (both rows have the same parents)
+    };
+    auto side = [&](int q) {
+      Side S;
+      const int z = z0 - 1 + q;
+      const bool inz = q < nz + 2 && z >= 0 && z < A.g.nz;
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
-        const bool in = inz && yr[e] >= 0 && yr[e] < A.g.ny;
-        float a = 0.f, b = 0.f, c = 0.f;
-        if (MODE == kUp && in) {
-          const float *q = A.y1 + (int64_t)A.nx1 * ((yr[e] >> 1) + (int64_t)A.ny1 * (z >> 1));
-          if (X < A.nx1) a = __ldg(q + X);
-          if (X + 1 < A.nx1) b = __ldg(q + X + 1);
-          if (rim) c = __ldg(q + (xr >> 1));
+        S.s[e] = S.a[e] = S.b[e] = 0.f;
+        if (inz && yin[e] && rim) {
+          const int64_t o = (int64_t)A.px * (yr[e] + (int64_t)A.g.ny * z) + xr;
+          S.s[e] = __ldg(A.s32 + o);
+          S.a[e] = __ldg(in1 + o);
+          if (MODE != kDown) S.b[e] = __ldg(in2 + o);
         }
-        const int64_t o = (int64_t)A.px * (yr[e] + (int64_t)A.g.ny * z);
-        R[e] = row0_load<MODE>(A, o + xl, in && act, a, b, beta, first);
-        ur[e] = rim0<MODE>(A, o + xr, in && rim, c, beta, first);
       }
+      S.y0 = S.y1 = S.yc = S.yh0 = S.yh1 = 0.f;
+      if (MODE == kUp && inz) {
+        const float *y = A.y1 + (int64_t)A.nx1 * A.ny1 * (z >> 1);
+        if (yin[0]) {
+          const float *q1 = y + (int64_t)A.nx1 * (yr[0] >> 1);
+          if (X < A.nx1) S.y0 = __ldg(q1 + X);
+          if (X + 1 < A.nx1) S.y1 = __ldg(q1 + X + 1);
+          if (rim) S.yc = __ldg(q1 + (xr >> 1));
+        }
+        if (hin) {
+          const float *q1 = y + (int64_t)A.nx1 * (yh >> 1);
+          if (X < A.nx1) S.yh0 = __ldg(q1 + X);
+          if (X + 1 < A.nx1) S.yh1 = __ldg(q1 + X + 1);
+        }
+      }
+      return S;
+    };
+    // sigma, v (and r, w) of the row at `at` of plane q from its inputs
+    auto row_of = [&](int q, int at, float y0, float y1) {
+      const float4 *src = sm3 + (q % kStages3) * 3 * kPlane3;
+      Row0 R;
+      R.s = src[at];
+      const float4 a = src[kPlane3 + at], b = src[2 * kPlane3 + at];
+      R.a = R.v = a;
+      if (MODE == kDown)
+        R.w = b;
+      else if (MODE == kUp)
+        R.v = make_float4(fmaf(b.x, y0, kOmega * a.x), fmaf(b.y, y0, kOmega * a.y),
+                          fmaf(b.z, y1, kOmega * a.z), fmaf(b.w, y1, kOmega * a.w));
+      else if (!first)
+        R.v = make_float4(fmaf(beta, b.x, a.x), fmaf(beta, b.y, a.y), fmaf(beta, b.z, a.z),
+                          fmaf(beta, b.w, a.w));
+      return R;
+    };
+    // the two rows of plane q, u of their rim node, and (planes with a place in
+    // us) u of the halo row
+    auto form = [&](int q, const Side &S, Row0 (&R)[2], float (&ur)[2], float4 *u) {
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        R[e] = row_of(q, pr[e], S.y0, S.y1);
+        if (MODE == kDown) ur[e] = S.s[e] * S.a[e];
+        else if (MODE == kUp) ur[e] = S.s[e] * fmaf(S.b[e], S.yc, kOmega * S.a[e]);
+        else ur[e] = S.s[e] * (first ? S.a[e] : fmaf(beta, S.b[e], S.a[e]));
+      }
+      if (edge && u) {
+        const Row0 H = row_of(q, ph, S.yh0, S.yh1);
+        u[ph] = mul4f(H.s, H.v);
+      }
+    };
+    auto landed = [] {   // the oldest plane in flight
+      asm volatile("cp.async.wait_group %0;" ::"n"(kStages3 - 1) : "memory");
     };
     Row0 C[2], N[2];
     float urc[2], urn[2];
     float4 um[2], uc[2];
-    load(z0 - 1, C, urc);
+#pragma unroll
+    for (int q = 0; q < kStages3; ++q) issue(q);
+    Side S = side(0), Sn = side(1);
+    landed();
+    form(0, S, C, urc, nullptr);
+    issue(kStages3);
 #pragma unroll
     for (int e = 0; e < 2; ++e) um[e] = mul4f(C[e].s, C[e].v);
-    load(z0, C, urc);
-    __syncthreads();   // the previous tile's planes are no longer read
+    S = Sn;
+    Sn = side(2);
+    landed();
+    __syncthreads();   // the previous tile's planes of u are no longer read
+    form(1, S, C, urc, us);
+    issue(kStages3 + 1);
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
       uc[e] = mul4f(C[e].s, C[e].v);
-      us[0][pr[e]][lane] = uc[e];
+      us[pr[e]] = uc[e];
     }
     float c0 = 0.f, c1 = 0.f;
     int cur = 0;
     for (int j = 0; j < nz; ++j) {
       const int z = z0 + j;
-      load(z + 1, N, urn);
+      S = Sn;
+      Sn = side(j + 3);
       const int nxt = (cur == 2) ? 0 : cur + 1;
+      landed();
+      form(j + 2, S, N, urn, us + nxt * kPlane3);
+      issue(j + 2 + kStages3);
       float4 un[2];
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
         un[e] = mul4f(N[e].s, N[e].v);
-        us[nxt][pr[e]][lane] = un[e];
+        us[nxt * kPlane3 + pr[e]] = un[e];
       }
       __syncthreads();
-      if (rows) {
+      {
         float fP = 1.f, fN = 1.f;
         if ((z & mask) == 0 && z > 0) fP = p2f(L.kc - __ldg(A.kx + crow - layer));
         if (((z + 1) & mask) == 0 && z + 1 < A.g.nz) fN = p2f(L.kc - __ldg(A.kx + crow + layer));
         const float hz = (half && (z == 0 || z == A.g.nz - 1)) ? 0.5f : 1.f;
-        const float4 yu = us[cur][pr[0] - 1][lane], yd = us[cur][pr[1] + 1][lane];
+        const float4 yu = us[cur * kPlane3 + pr[0] - 32], yd = us[cur * kPlane3 + pr[1] + 32];
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
           float uL = __shfl_up_sync(0xffffffffu, uc[e].w, 1);
@@ -793,13 +902,13 @@ k_mg0_3d(const Mg0 A, int tiles_x, int tiles_y, int zc, int ntiles, MgCtl *ctl, 
             const float zs = fmaf(f4(um[e], i), fP, f4(un[e], i) * fN);
             off[i] = f4(C[e].s, i) * fmaf(wx, xs[i], L.hx[i] * fmaf(hz, ys, hy[e] * zs));
           }
-          if (act && yr[e] < A.g.ny) {
+          if (act && yin[e]) {
             const int64_t o = (int64_t)A.px * (yr[e] + (int64_t)A.g.ny * z) + xl;
             dot += row0_out<MODE>(A, o, C[e], off, L.wd, c0, c1);
           }
         }
         if (MODE == kDown && ((j & 1) || j == nz - 1)) {
-          if (yr[0] < A.g.ny)
+          if (yin[0])
             coarse_out(A, (int64_t)A.nx1 * ((yr[0] >> 1) + (int64_t)A.ny1 * (z >> 1)), X, c0, c1);
           c0 = c1 = 0.f;
         }
@@ -813,6 +922,9 @@ k_mg0_3d(const Mg0 A, int tiles_x, int tiles_y, int zc, int ntiles, MgCtl *ctl, 
       }
       cur = nxt;
     }
+    // (copies past the last plane are zero fills of unused stages; they have
+    // to land before the next tile issues into them)
+    asm volatile("cp.async.wait_all;" ::: "memory");
   }
   if (MODE != kDown) dot0_end<MODE>(dot, ctl, part);
 }
@@ -1009,6 +1121,18 @@ eik_status mg_create(MgState **out, const Grid &g, const CellGrid &cg, int px, i
     g_msg = "multigrid: device allocation failed";
     return EIK_ERR_OOM;
   }
+  if (g.ndim == 3 &&
+      (cudaFuncSetAttribute(k_mg0_3d<kDown>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                            (int)kSmem3) != cudaSuccess ||
+       cudaFuncSetAttribute(k_mg0_3d<kUp>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                            (int)kSmem3) != cudaSuccess ||
+       cudaFuncSetAttribute(k_mg0_3d<kDir>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                            (int)kSmem3) != cudaSuccess)) {
+    cudaGetLastError();
+    mg_destroy(mg);
+    g_msg = "multigrid: cannot reserve shared memory";
+    return EIK_ERR_CUDA;
+  }
   *out = mg;
   return EIK_OK;
 }
@@ -1092,7 +1216,7 @@ static void launch0(MgState *mg, const MgFine &f, int set, cudaStream_t s) {
     int zc = 16;
     while (zc > 2 && (int64_t)tx * ty * ((g.nz + zc - 1) / zc) < mg->cap / 4) zc /= 2;
     const int64_t nt = (int64_t)tx * ty * ((g.nz + zc - 1) / zc);
-    k_mg0_3d<MODE><<<(int)std::min<int64_t>(nt, mg->cap), kThreads3, 0, s>>>(
+    k_mg0_3d<MODE><<<(int)std::min<int64_t>(nt, mg->cap), kThreads3, kSmem3, s>>>(
         a, tx, ty, zc, (int)nt, mg->ctl, mg->part);
   }
 }
