@@ -6,17 +6,29 @@
 // Green's function K_0(f~|x|/hbar) / (2 pi hbar^2) (Eq. GreensFunction2D);
 // S = -hbar log phi.  Every convolution is the linear one over the grid,
 // computed by complex FP64 transforms of arrays zero-padded to P_a >= 2 n_a - 1
-// points per axis (powers of two) with the kernel sampled at the offsets
+// points per axis with the kernel sampled at the offsets
 // -(n_a - 1) .. n_a - 1 and wrapped; G's sample at the origin is its average
 // over the grid cell.
 //
-// Transforms: a 2D transform is a pass of 1D transforms along the rows, a
-// tiled transpose, and a second row pass; the spectrum stays in the
-// transposed layout, where the pointwise products are taken, and the inverse
-// retraces the same steps.  A row transform runs in one block, in shared
-// memory, as the Stockham self-sorting form of the mixed-radix FFT: lengths
-// P = 2^a 3^b 5^c (the smallest >= 2n - 1), stages of radix 4, 2, 3 and 5,
-// each reading one buffer and writing the other in natural order.
+// Transforms.  Everything transformed is real, so two rows of a grid function
+// travel as the real and imaginary part of one complex row, and only the
+// columns kx <= P_x / 2 of its spectrum are kept.  One term is four launches:
+//   k_rows_x  inverse row transforms of the last product, which give the term
+//             (added to phi); psi of the next term; its forward transforms
+//   k_unpack  split of the row pairs' spectra, transposed
+//   k_cols    forward column transform, times the kernel's spectrum, inverse
+//   k_repack  the row pairs' spectra again, transposed back
+// Both kernels are even in x and y: their spectra are real, and their row
+// pairs' and column pairs' transforms need no split.  Against complex
+// transforms of the whole padded array (two row passes each way, products,
+// embedding and extraction as passes of their own) this does half of the FP64
+// work, which is what bounds the series on this GPU, and a third of the
+// launches: 513^2, six terms 3.65 ms before, 2.05 ms now.
+//
+// A row transform runs in one block, in shared memory, as the Stockham
+// self-sorting form of the mixed-radix FFT: lengths P = 2^a 3^b 5^c (the
+// smallest >= 2n - 1), stages of radix 4, 2, 3 and 5, each reading one buffer
+// and writing the other in natural order.
 //
 // K_0 and K_1 come from their integral representation
 // K_nu(x) = int_0^inf exp(-x cosh t) cosh(nu t) dt (DLMF 10.32.9), summed by
@@ -136,7 +148,7 @@ __device__ __forceinline__ void stockham_stage(const double2 *x, double2 *y, int
     for (int r = 0; r < R; ++r) {
       double2 t = x[j + r * m];
       if (r > 0 && k > 0) {
-        double2 w = tw[(r * k * tstep) % P];
+        double2 w = __ldg(tw + r * k * tstep);   // r k tstep < P
         if (INV) w.y = -w.y;
         t = cmul(w, t);
       }
@@ -149,14 +161,11 @@ __device__ __forceinline__ void stockham_stage(const double2 *x, double2 *y, int
   }
 }
 
+// Transform of the row in x (y: scratch of the same length); returns the
+// buffer that holds the result.  Every stage ends with a barrier.
 template <bool INV>
-__global__ void k_fft_rows(double2 *a, int P, Radices rad, DftConst kc,
-                           const double2 *__restrict__ tw) {
-  extern __shared__ double2 fsm[];
-  double2 *x = fsm, *y = fsm + P;
-  double2 *row = a + (size_t)blockIdx.x * P;
-  for (int i = threadIdx.x; i < P; i += blockDim.x) x[i] = row[i];
-  __syncthreads();
+__device__ __forceinline__ double2 *fft_row(double2 *x, double2 *y, int P, const Radices &rad,
+                                            const DftConst &kc, const double2 *__restrict__ tw) {
   int Ns = 1;
   for (int st = 0; st < rad.n; ++st) {
     const int R = rad.r[st];
@@ -172,24 +181,132 @@ __global__ void k_fft_rows(double2 *a, int P, Radices rad, DftConst kc,
     y = tmp;
     Ns *= R;
   }
-  for (int i = threadIdx.x; i < P; i += blockDim.x) row[i] = x[i];
+  return x;
 }
 
-// out (cols x rows) = transpose of in (rows x cols), 32 x 32 tiles.
-__global__ void k_transpose(const double2 *__restrict__ in, double2 *__restrict__ out, int rows,
-                            int cols) {
-  __shared__ double2 t[32][33];
-  const int x = blockIdx.x * 32 + threadIdx.x;
-  for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-    const int y = blockIdx.y * 32 + k;
-    if (x < cols && y < rows) t[k][threadIdx.x] = in[(size_t)y * cols + x];
+// Rows 2 b and 2 b + 1 of the grid (block b).  INV: inverse transforms of Z's
+// row, scaled, give the term's rows; phi = v, or phi += sign v.  FWD: forward
+// transforms of psi = (f^2 - f~^2) v (Table 1 step 9), or of the grid function
+// `in` itself, into Z's row.
+template <bool INV, bool FWD>
+__global__ void k_rows_x(double2 *Z, int P, Radices rad, DftConst kc,
+                         const double2 *__restrict__ tw, int nx, int ny,
+                         const double *__restrict__ in, const double *__restrict__ f, double ft2,
+                         double scale, double sign, int first, double *__restrict__ phi) {
+  extern __shared__ double2 fsm[];
+  double2 *x = fsm, *y = fsm + P;
+  double2 *row = Z + (size_t)blockIdx.x * P;
+  const int64_t o0 = (int64_t)2 * blockIdx.x * nx, o1 = o0 + nx;
+  const bool two = 2 * blockIdx.x + 1 < ny;
+  if (INV) {
+    for (int i = threadIdx.x; i < P; i += blockDim.x) x[i] = row[i];
+    __syncthreads();
+    double2 *z = fft_row<true>(x, y, P, rad, kc, tw);
+    if (z != x) {
+      y = x;
+      x = z;
+    }
+    for (int i = threadIdx.x; i < P; i += blockDim.x) {
+      double2 psi = make_double2(0.0, 0.0);
+      if (i < nx) {
+        const double v0 = scale * x[i].x, v1 = scale * x[i].y;
+        phi[o0 + i] = first ? v0 : phi[o0 + i] + sign * v0;
+        if (two) phi[o1 + i] = first ? v1 : phi[o1 + i] + sign * v1;
+        if (FWD) {
+          const double f0 = f[o0 + i];
+          psi.x = (f0 * f0 - ft2) * v0;
+          if (two) {
+            const double f1 = f[o1 + i];
+            psi.y = (f1 * f1 - ft2) * v1;
+          }
+        }
+      }
+      if (FWD) x[i] = psi;
+    }
+  } else {
+    for (int i = threadIdx.x; i < P; i += blockDim.x)
+      x[i] = (i < nx) ? make_double2(in[o0 + i], two ? in[o1 + i] : 0.0) : make_double2(0.0, 0.0);
+  }
+  if (!FWD) return;
+  __syncthreads();
+  const double2 *z = fft_row<false>(x, y, P, rad, kc, tw);
+  for (int i = threadIdx.x; i < P; i += blockDim.x) row[i] = z[i];
+}
+
+// B[k][y] (hx x ny), the spectrum of grid row y at kx = k, from the row pairs'
+// transforms Z (Z_k = A_k + i B_k with A, B Hermitian): 32 x 32 tiles of (k,
+// pair), transposed through shared memory.
+__global__ void k_unpack(const double2 *__restrict__ Z, double2 *__restrict__ B, int P, int hx,
+                         int ny) {
+  __shared__ double2 t[32][33], u[32][33];
+  const int k = blockIdx.x * 32 + threadIdx.x, np = (ny + 1) / 2;
+  for (int q = threadIdx.y; q < 32; q += blockDim.y) {
+    const int r = blockIdx.y * 32 + q;
+    if (k < hx && r < np) {
+      const double2 a = Z[(size_t)r * P + k], b = Z[(size_t)r * P + (k == 0 ? 0 : P - k)];
+      t[q][threadIdx.x] = make_double2(0.5 * (a.x + b.x), 0.5 * (a.y - b.y));
+      u[q][threadIdx.x] = make_double2(0.5 * (a.y + b.y), 0.5 * (b.x - a.x));
+    }
   }
   __syncthreads();
-  const int ox = blockIdx.y * 32 + threadIdx.x;
-  for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-    const int oy = blockIdx.x * 32 + k;
-    if (ox < rows && oy < cols) out[(size_t)oy * rows + ox] = t[threadIdx.x][k];
+  // rows of B: columns y = 2 r and 2 r + 1 side by side
+  const int y = blockIdx.y * 64 + 2 * threadIdx.x;
+  for (int q = threadIdx.y; q < 32; q += blockDim.y) {
+    const int kk = blockIdx.x * 32 + q;
+    if (kk < hx) {
+      if (y < ny) B[(size_t)kk * ny + y] = t[threadIdx.x][q];
+      if (y + 1 < ny) B[(size_t)kk * ny + y + 1] = u[threadIdx.x][q];
+    }
   }
+}
+
+// The inverse of k_unpack: Z_k = A_k + i B_k, also for kx > P / 2 by symmetry.
+__global__ void k_repack(const double2 *__restrict__ B, double2 *__restrict__ Z, int P, int hx,
+                         int ny) {
+  __shared__ double2 t[32][33], u[32][33];
+  const int y = blockIdx.y * 64 + 2 * threadIdx.x, np = (ny + 1) / 2;
+  for (int q = threadIdx.y; q < 32; q += blockDim.y) {
+    const int kk = blockIdx.x * 32 + q;
+    if (kk < hx) {
+      t[q][threadIdx.x] = (y < ny) ? B[(size_t)kk * ny + y] : make_double2(0.0, 0.0);
+      u[q][threadIdx.x] = (y + 1 < ny) ? B[(size_t)kk * ny + y + 1] : make_double2(0.0, 0.0);
+    }
+  }
+  __syncthreads();
+  const int k = blockIdx.x * 32 + threadIdx.x;
+  for (int q = threadIdx.y; q < 32; q += blockDim.y) {
+    const int r = blockIdx.y * 32 + q;
+    if (k < hx && r < np) {
+      const double2 a = t[threadIdx.x][q], b = u[threadIdx.x][q];
+      Z[(size_t)r * P + k] = make_double2(a.x - b.y, a.y + b.x);
+      if (k > 0 && P - k >= hx) Z[(size_t)r * P + P - k] = make_double2(a.x + b.y, b.x - a.y);
+    }
+  }
+}
+
+// One column kx = blockIdx.x of the spectrum: forward transform along y (zero
+// past the grid), times the kernel's spectrum, inverse.
+__global__ void k_cols(double2 *B, int P, Radices rad, DftConst kc,
+                       const double2 *__restrict__ tw, int ny, const double *__restrict__ K) {
+  extern __shared__ double2 fsm[];
+  double2 *x = fsm, *y = fsm + P;
+  double2 *row = B + (size_t)blockIdx.x * ny;
+  const double *k = K + (size_t)blockIdx.x * P;
+  for (int i = threadIdx.x; i < P; i += blockDim.x)
+    x[i] = (i < ny) ? row[i] : make_double2(0.0, 0.0);
+  __syncthreads();
+  double2 *z = fft_row<false>(x, y, P, rad, kc, tw);
+  if (z != x) {
+    y = x;
+    x = z;
+  }
+  for (int i = threadIdx.x; i < P; i += blockDim.x) {
+    const double m = k[i];
+    x[i] = make_double2(m * x[i].x, m * x[i].y);
+  }
+  __syncthreads();
+  z = fft_row<true>(x, y, P, rad, kc, tw);
+  for (int i = threadIdx.x; i < ny; i += blockDim.x) row[i] = z[i];
 }
 
 // K_nu(x), nu = 0 or 1, x > 0 (integral representation, trapezoidal rule).
@@ -215,20 +332,6 @@ __device__ double bessel_k(int nu, double x) {
   return eta * ex * sum;
 }
 
-// Wrapped offset of index i of a transform of length P for an axis of n
-// nodes: offsets 0 .. n-1 at i = 0 .. n-1, -1 .. -(n-1) at P-1 .. P-n+1.
-__device__ __forceinline__ bool wrapped(int i, int P, int n, int *o) {
-  if (i < n) {
-    *o = i;
-    return true;
-  }
-  if (i >= P - (n - 1)) {
-    *o = i - P;
-    return true;
-  }
-  return false;
-}
-
 // G at the offsets 0 <= b <= a < m, packed as tab[a (a + 1) / 2 + b] (G
 // depends on |offset| only, so one octant serves all); the origin takes *g0.
 __global__ void k_green_table(double *tab, int m, double h, double ft, double hbar,
@@ -245,25 +348,54 @@ __global__ void k_green_table(double *tab, int m, double h, double ft, double hb
   }
 }
 
-// Kernel sampled at the wrapped offsets into a (Py x Px, pitch Px) complex
-// array: mode 0 G~ = exp(-f~ r / hbar); mode 1 G from the octant table.
-__global__ void k_fill_kernel(double2 *a, int Px, int Py, int nx, int ny, double h, double ft,
-                              double hbar, int mode, const double *__restrict__ tab) {
-  const int64_t tot = (int64_t)Px * Py;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < tot;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int ix = (int)(e % Px), iy = (int)(e / Px);
-    int ox, oy;
-    double v = 0.0;
-    if (wrapped(ix, Px, nx, &ox) && wrapped(iy, Py, ny, &oy)) {
-      if (mode == 0) {
-        v = exp(-ft * h * hypot((double)ox, (double)oy) / hbar);
-      } else {
-        const int p = max(abs(ox), abs(oy)), q = min(abs(ox), abs(oy));
-        v = tab[(int64_t)p * (p + 1) / 2 + q];
-      }
-    }
-    a[e] = make_double2(v, 0.0);
+// Kernel rows y = 2 b and 2 b + 1 (y >= 0 offsets) at the wrapped x offsets:
+// mode 0 G~ = exp(-f~ r / hbar), mode 1 G from the octant table.  Both rows are
+// even in x, so the pair's transform holds their real spectra as its real and
+// imaginary part: KX[y][kx], kx < hx.
+__global__ void k_kernel_rows(double *__restrict__ KX, int P, Radices rad, DftConst kc,
+                              const double2 *__restrict__ tw, int nx, int ny, int hx, double h,
+                              double ft, double hbar, int mode, const double *__restrict__ tab) {
+  extern __shared__ double2 fsm[];
+  const int y0 = 2 * blockIdx.x;
+  auto value = [&](int ox, int oy) {
+    if (mode == 0) return exp(-ft * h * hypot((double)ox, (double)oy) / hbar);
+    const int p = max(abs(ox), abs(oy)), q = min(abs(ox), abs(oy));
+    return tab[(int64_t)p * (p + 1) / 2 + q];
+  };
+  // the half x >= 0; the other half is its mirror image
+  for (int i = threadIdx.x; i < nx; i += blockDim.x) {
+    const double2 v = make_double2(value(i, y0), (y0 + 1 < ny) ? value(i, y0 + 1) : 0.0);
+    fsm[i] = v;
+    if (i > 0) fsm[P - i] = v;
+  }
+  for (int i = nx + threadIdx.x; i < P - nx + 1; i += blockDim.x) fsm[i] = make_double2(0.0, 0.0);
+  __syncthreads();
+  const double2 *z = fft_row<false>(fsm, fsm + P, P, rad, kc, tw);
+  for (int i = threadIdx.x; i < hx; i += blockDim.x) {
+    KX[(size_t)y0 * hx + i] = z[i].x;
+    if (y0 + 1 < ny) KX[(size_t)(y0 + 1) * hx + i] = z[i].y;
+  }
+}
+
+// Columns kx = 2 b and 2 b + 1 of the kernel's spectrum, likewise: K[kx][ky].
+__global__ void k_kernel_cols(const double *__restrict__ KX, double *__restrict__ K, int P,
+                              Radices rad, DftConst kc, const double2 *__restrict__ tw, int ny,
+                              int hx) {
+  extern __shared__ double2 fsm[];
+  const int k0 = 2 * blockIdx.x;
+  const bool two = k0 + 1 < hx;
+  for (int i = threadIdx.x; i < ny; i += blockDim.x) {
+    const double *q = KX + (size_t)i * hx + k0;
+    const double2 v = make_double2(q[0], two ? q[1] : 0.0);
+    fsm[i] = v;
+    if (i > 0) fsm[P - i] = v;
+  }
+  for (int i = ny + threadIdx.x; i < P - ny + 1; i += blockDim.x) fsm[i] = make_double2(0.0, 0.0);
+  __syncthreads();
+  const double2 *z = fft_row<false>(fsm, fsm + P, P, rad, kc, tw);
+  for (int i = threadIdx.x; i < P; i += blockDim.x) {
+    K[(size_t)k0 * P + i] = z[i].x;
+    if (two) K[(size_t)(k0 + 1) * P + i] = z[i].y;
   }
 }
 
@@ -296,50 +428,10 @@ __global__ void k_cell_average(const double *__restrict__ val, double h, double 
   }
 }
 
-// Pointwise spectral product b *= k.
-__global__ void k_cmul(double2 *b, const double2 *__restrict__ k, int64_t n) {
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-       e += (int64_t)gridDim.x * blockDim.x)
-    b[e] = cmul(b[e], k[e]);
-}
-
-// Zero-padded complex array of psi = (f^2 - f~^2) g for the grid function g
-// (Table 1 step 9), zero outside the grid.
-__global__ void k_embed(double2 *a, int Px, int Py, int nx, int ny, const double *__restrict__ f,
-                        double ft2, const double *__restrict__ g) {
-  const int64_t tot = (int64_t)Px * Py;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < tot;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int ix = (int)(e % Px), iy = (int)(e / Px);
-    double v = 0.0;
-    if (ix < nx && iy < ny) {
-      const int64_t i = (int64_t)iy * nx + ix;
-      const double fi = f[i];
-      v = (fi * fi - ft2) * g[i];   // psi_i = (f^2 - f~^2) phi_{i-1}
-    }
-    a[e] = make_double2(v, 0.0);
-  }
-}
-
-__global__ void k_delta(double2 *a, int Px, const int64_t *__restrict__ src, int64_t nsrc, int nx) {
+// The sources' Kronecker deltas on the grid (zeroed before).
+__global__ void k_delta(double *a, const int64_t *__restrict__ src, int64_t nsrc) {
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= nsrc) return;
-  const int64_t j = src[k];
-  const int x = (int)(j % nx), y = (int)(j / nx);
-  a[(size_t)y * Px + x] = make_double2(1.0, 0.0);
-}
-
-// Grid values of an inverse transform: term = scale * Re(a); phi += sign term.
-__global__ void k_extract(const double2 *__restrict__ a, int Px, int nx, int64_t n, double scale,
-                          double sign, double *__restrict__ term, double *__restrict__ phi,
-                          int first) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int x = (int)(i % nx), y = (int)(i / nx);
-    const double v = scale * a[(size_t)y * Px + x].x;
-    term[i] = v;
-    phi[i] = first ? v : phi[i] + sign * v;
-  }
+  if (k < nsrc) a[src[k]] = 1.0;
 }
 
 __global__ void k_log(const double *__restrict__ phi, int64_t n, double hbar, double *S) {
@@ -376,11 +468,14 @@ __global__ void k_fminmax(const double *__restrict__ f, int64_t n, double *out, 
 }
 
 struct Fft2 {
-  int Px, Py;
+  int Px, Py, hx;   // transform lengths; columns of the spectrum kept
+  int nx, ny;
   Radices rx, ry;
   DftConst kc;
   double2 *twx, *twy;
-  double2 *A, *B;   // A: Py x Px (grid layout); B: Px x Py (transposed)
+  double2 *Z;       // row pairs: ceil(ny / 2) x Px
+  double2 *B;       // spectrum by column: hx x ny
+  double *KX, *K;   // kernel: rows' spectra ny x hx, spectrum hx x Py
   cudaStream_t s;
 };
 
@@ -411,36 +506,38 @@ Radices radices(int P) {
   return r;
 }
 
-void rows(const Fft2 &F, double2 *a, int count, int P, const Radices &rad, const double2 *tw,
-          bool inv) {
-  const int th = std::min(512, std::max(32, P / 2));
-  const size_t sm = 2 * sizeof(double2) * P;
-  if (inv)
-    k_fft_rows<true><<<count, th, sm, F.s>>>(a, P, rad, F.kc, tw);
-  else
-    k_fft_rows<false><<<count, th, sm, F.s>>>(a, P, rad, F.kc, tw);
+int fft_threads(int P) { return std::min(512, std::max(32, P / 2)); }
+size_t fft_smem(int P) { return 2 * sizeof(double2) * P; }
+
+// Spectrum of a kernel into F.K.
+void kernel_spectrum(const Fft2 &F, double h, double ft, double hbar, int mode, const double *tab) {
+  k_kernel_rows<<<(F.ny + 1) / 2, fft_threads(F.Px), fft_smem(F.Px), F.s>>>(
+      F.KX, F.Px, F.rx, F.kc, F.twx, F.nx, F.ny, F.hx, h, ft, hbar, mode, tab);
+  k_kernel_cols<<<(F.hx + 1) / 2, fft_threads(F.Py), fft_smem(F.Py), F.s>>>(
+      F.KX, F.K, F.Py, F.ry, F.kc, F.twy, F.ny, F.hx);
 }
 
-void transpose(const Fft2 &F, const double2 *in, double2 *out, int r, int c) {
-  dim3 g((c + 31) / 32, (r + 31) / 32), b(32, 8);
-  k_transpose<<<g, b, 0, F.s>>>(in, out, r, c);
+// Z (forward row transforms) -> Z (before the inverse ones), times F.K.
+void convolve(const Fft2 &F) {
+  const dim3 g((F.hx + 31) / 32, ((F.ny + 1) / 2 + 31) / 32), b(32, 8);
+  k_unpack<<<g, b, 0, F.s>>>(F.Z, F.B, F.Px, F.hx, F.ny);
+  k_cols<<<F.hx, fft_threads(F.Py), fft_smem(F.Py), F.s>>>(F.B, F.Py, F.ry, F.kc, F.twy, F.ny, F.K);
+  k_repack<<<g, b, 0, F.s>>>(F.B, F.Z, F.Px, F.hx, F.ny);
 }
 
-// A (grid layout) -> B (spectrum, transposed layout).  Rows of A at and past
-// `rows_in` are zero (grid functions), so their transforms are zero and are
-// skipped.
-void forward(const Fft2 &F, int rows_in) {
-  rows(F, F.A, rows_in, F.Px, F.rx, F.twx, false);
-  transpose(F, F.A, F.B, F.Py, F.Px);
-  rows(F, F.B, F.Px, F.Py, F.ry, F.twy, false);
+template <bool INV, bool FWD>
+void rows_x(const Fft2 &F, const double *in, const double *f, double ft2, double scale,
+            double sign, int first, double *phi) {
+  k_rows_x<INV, FWD><<<(F.ny + 1) / 2, fft_threads(F.Px), fft_smem(F.Px), F.s>>>(
+      F.Z, F.Px, F.rx, F.kc, F.twx, F.nx, F.ny, in, f, ft2, scale, sign, first, phi);
 }
 
-// B (spectrum) -> A (grid layout), unscaled; only the first `rows_out` rows
-// of A (the grid's) are transformed back.
-void inverse(const Fft2 &F, int rows_out) {
-  rows(F, F.B, F.Px, F.Py, F.ry, F.twy, true);
-  transpose(F, F.B, F.A, F.Px, F.Py);
-  rows(F, F.A, rows_out, F.Px, F.rx, F.twx, true);
+// The attribute belongs to the function: always the largest row, so that
+// concurrent calls agree.
+template <class Kn>
+bool max_smem(Kn *fn) {
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)fft_smem(kMaxFft)) == cudaSuccess;
 }
 
 // Work arrays from the stream-ordered allocator (the device's memory pool):
@@ -498,30 +595,29 @@ extern "C" eik_status eik_fft_series(const int64_t *dims, double h, double hbar,
                   std::sqrt(0.125 * (5.0 + std::sqrt(5.0))),
                   std::sqrt(0.125 * (5.0 - std::sqrt(5.0)))};
   F.s = s;
-  const int64_t np = (int64_t)F.Px * F.Py;
+  F.nx = nx;
+  F.ny = ny;
+  F.hx = F.Px / 2 + 1;
   Buf buf(s);
-  double2 *K = nullptr;
-  double *fd = nullptr, *phi = nullptr, *t0 = nullptr, *t1 = nullptr, *mm = nullptr, *g0 = nullptr;
+  double *fd = nullptr, *phi = nullptr, *Sd = nullptr, *mm = nullptr, *g0 = nullptr;
   double *gtab = nullptr, *cval = nullptr;
   const int m = std::max(nx, ny);
   int64_t *src = nullptr;
   int *bad = nullptr;
-  if (!buf.get(&F.twx, F.Px) || !buf.get(&F.twy, F.Py) || !buf.get(&F.A, np) ||
-      !buf.get(&F.B, np) || !buf.get(&K, np) || !buf.get(&fd, n) || !buf.get(&phi, n) ||
-      !buf.get(&t0, n) || !buf.get(&t1, n) || !buf.get(&mm, 2) || !buf.get(&g0, 1) ||
+  if (!buf.get(&F.twx, F.Px) || !buf.get(&F.twy, F.Py) ||
+      !buf.get(&F.Z, (size_t)((ny + 1) / 2) * F.Px) || !buf.get(&F.B, (size_t)F.hx * ny) ||
+      !buf.get(&F.KX, (size_t)F.hx * ny) || !buf.get(&F.K, (size_t)F.hx * F.Py) ||
+      !buf.get(&fd, n) || !buf.get(&phi, n) || !buf.get(&Sd, n) || !buf.get(&mm, 2) ||
+      !buf.get(&g0, 1) ||
       !buf.get(&src, nsrc) || !buf.get(&bad, 1) ||
       !buf.get(&gtab, (size_t)m * (m + 1) / 2) || !buf.get(&cval, kSimpson + 1)) {
     cudaGetLastError();
     return EIK_ERR_OOM;
   }
-  for (int P : {F.Px, F.Py}) {
-    const size_t sm = 2 * sizeof(double2) * P;
-    if (cudaFuncSetAttribute(k_fft_rows<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)std::max<size_t>(sm, 48 * 1024)) != cudaSuccess ||
-        cudaFuncSetAttribute(k_fft_rows<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)std::max<size_t>(sm, 48 * 1024)) != cudaSuccess)
-      return EIK_ERR_CUDA;
-  }
+  if (!max_smem(k_rows_x<false, true>) || !max_smem(k_rows_x<true, true>) ||
+      !max_smem(k_rows_x<true, false>) || !max_smem(k_cols) || !max_smem(k_kernel_rows) ||
+      !max_smem(k_kernel_cols))
+    return EIK_ERR_CUDA;
   const int nb = 152 * 8;
   if (cudaMemcpyAsync(fd, f, sizeof(double) * n, cudaMemcpyDefault, s) != cudaSuccess ||
       cudaMemcpyAsync(src, hs.data(), sizeof(int64_t) * nsrc, cudaMemcpyHostToDevice, s) !=
@@ -544,39 +640,30 @@ extern "C" eik_status eik_fft_series(const int64_t *dims, double h, double hbar,
   k_twiddles<<<(F.Px + 255) / 256, 256, 0, s>>>(F.twx, F.Px);
   k_twiddles<<<(F.Py + 255) / 256, 256, 0, s>>>(F.twy, F.Py);
   const double inv = 1.0 / ((double)F.Px * F.Py);
-  // Table 1 steps 1-5: phi_0 = G~ * delta_kron
-  k_fill_kernel<<<nb, kThreads, 0, s>>>(F.A, F.Px, F.Py, nx, ny, h, ft, hbar, 0, gtab);
-  forward(F, F.Py);
-  cudaMemcpyAsync(K, F.B, sizeof(double2) * np, cudaMemcpyDeviceToDevice, s);
-  cudaMemsetAsync(F.A, 0, sizeof(double2) * np, s);
-  k_delta<<<(int)((nsrc + 255) / 256), 256, 0, s>>>(F.A, F.Px, src, nsrc, nx);
-  forward(F, ny);
-  k_cmul<<<nb, kThreads, 0, s>>>(F.B, K, np);
-  inverse(F, ny);
-  // step 6: phi = phi_0 (t0 holds phi_{i-1})
-  k_extract<<<nb, kThreads, 0, s>>>(F.A, F.Px, nx, n, inv, 1.0, t0, phi, 1);
-  // step 7: transform of G
-  if (terms > 0) {
+  // Table 1 steps 1-6: phi = phi_0 = G~ * delta_kron (Sd holds the deltas)
+  kernel_spectrum(F, h, ft, hbar, 0, nullptr);
+  cudaMemsetAsync(Sd, 0, sizeof(double) * n, s);
+  k_delta<<<(int)((nsrc + 255) / 256), 256, 0, s>>>(Sd, src, nsrc);
+  rows_x<false, true>(F, Sd, nullptr, 0.0, 0.0, 0.0, 0, nullptr);
+  convolve(F);
+  if (terms == 0) {
+    rows_x<true, false>(F, nullptr, nullptr, 0.0, inv, 1.0, 1, phi);
+  } else {
+    rows_x<true, true>(F, nullptr, fd, ft * ft, inv, 1.0, 1, phi);
+    // step 7: transform of G
     k_cell_samples<<<(kSimpson + 1 + 63) / 64, 64, 0, s>>>(h, ft, hbar, cval);
     k_cell_average<<<1, kThreads, 0, s>>>(cval, h, hbar, g0);
     k_green_table<<<nb, kThreads, 0, s>>>(gtab, m, h, ft, hbar, g0);
-    k_fill_kernel<<<nb, kThreads, 0, s>>>(F.A, F.Px, F.Py, nx, ny, h, ft, hbar, 1, gtab);
-    forward(F, F.Py);
-    cudaMemcpyAsync(K, F.B, sizeof(double2) * np, cudaMemcpyDeviceToDevice, s);
+    kernel_spectrum(F, h, ft, hbar, 1, gtab);
+    // steps 8-14
+    for (int i = 1; i <= terms; ++i) {
+      convolve(F);
+      const double sign = (i & 1) ? -1.0 : 1.0;
+      if (i < terms) rows_x<true, true>(F, nullptr, fd, ft * ft, inv * h * h, sign, 0, phi);
+      else rows_x<true, false>(F, nullptr, nullptr, 0.0, inv * h * h, sign, 0, phi);
+    }
   }
-  // steps 8-14
-  double *prev = t0, *cur = t1;
-  for (int i = 1; i <= terms; ++i) {
-    k_embed<<<nb, kThreads, 0, s>>>(F.A, F.Px, F.Py, nx, ny, fd, ft * ft, prev);
-    forward(F, ny);
-    k_cmul<<<nb, kThreads, 0, s>>>(F.B, K, np);
-    inverse(F, ny);
-    k_extract<<<nb, kThreads, 0, s>>>(F.A, F.Px, nx, n, inv * h * h, (i & 1) ? -1.0 : 1.0, cur,
-                                      phi, 0);
-    std::swap(prev, cur);
-  }
-  // step 15 (into the buffer no longer needed)
-  double *Sd = cur;
+  // step 15
   k_log<<<nb, kThreads, 0, s>>>(phi, n, hbar, Sd);
   if (cudaGetLastError() != cudaSuccess) return EIK_ERR_CUDA;
   if (cudaMemcpyAsync(S_out, Sd, sizeof(double) * n, cudaMemcpyDefault, s) != cudaSuccess)
