@@ -74,7 +74,6 @@ struct MixCtl {
   int stalled;       // 1: the recurrence lost positivity: the solve ended early;
                      // 2: the residual grew too far, drop the correction
   int fault;         // a bounded device-side wait expired
-  float conj2;       // resident inner CG: 2 beta <p, A p_old> of the next direction
   int withhold;      // test hook: one warp never gets its first copy
   // packed batches (the single-grid passes ignore these)
   int first;         // the next pass is the inner solve's first (w = A r only)

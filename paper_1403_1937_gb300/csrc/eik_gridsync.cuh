@@ -30,10 +30,11 @@ constexpr unsigned long long kSyncWaitNs = 1000ull * 1000 * 1000;   // 1 s
 
 // Partials per exchange and block, and most blocks that take part (a warp
 // reads five slots per lane).
-constexpr int kSyncVals = 2;
+constexpr int kSyncVals = 3;
 constexpr int kSyncBlocks = 160;
-// A solver's buffer: the counter in a 128-byte line, then the slots.  The
-// counter is zeroed before every launch.
+// A solver's buffer: a 128-byte line with the counter (its first 32 bits,
+// zeroed before every launch) and, from the second word on, what a solver keeps
+// between launches; then the slots.
 constexpr int kSyncSlot0 = 16;
 constexpr size_t kSyncBytes =
     sizeof(unsigned long long) * (kSyncSlot0 + 2 * kSyncVals * kSyncBlocks);

@@ -798,7 +798,6 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
     // so from their first pass's maximum)
     st.dF = m->res.ok ? std::max(-126, std::min(126, std::ilogb(st.r_inf))) : 0;
     st.fd = st.rho_s;
-    st.conj2 = 0.f;
     st.iter = 0;
     st.done = 0;
     st.status = 0;
@@ -839,7 +838,7 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
         for (auto &e : m->ev) MCK(cudaEventCreate(&e));
       if (m->profile) MCK(cudaEventRecord(m->ev[0], s));
       // (the resident kernel starts from the residual's <r, r>; it has no
-      // initial pass of its own)
+      // initial pass of its own, and the count below is of inner solves)
       if (!m->res.ok) cg32_init(m->plan, g, m->cg, m->bufs, 0, s);
       m->launches[3]++;
       MCK(cudaGetLastError());
@@ -868,6 +867,7 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
             continue;
           }
           MCK(e);
+          m->launches[4]++;
           if (m->profile) MCK(cudaEventRecord(m->ev[2], s));
         } else if (m->profile) {
           // one timed iteration per host check: no launch runs past convergence
@@ -883,12 +883,11 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
         MCK(cudaStreamSynchronize(s));
         const int done_now = m->h_st->iter - before;   // of the resident kernel's launch
         before = m->h_st->iter;
-        if (m->res.ok) m->launches[4] += done_now;
         if (m->profile) {
           float t = 0.f;
           MCK(cudaEventElapsedTime(&t, m->ev[1], m->ev[2]));
           m->ms[4] += t;
-          m->timed[4] += m->res.ok ? done_now : 1;
+          m->timed[4] += m->res.ok ? done_now : 1;   // times are per iteration
         }
         if (m->h_st->done) break;
       }

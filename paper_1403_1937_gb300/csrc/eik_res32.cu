@@ -112,7 +112,7 @@ template <int kT, int ROWS, bool DREG>
 __global__ void __launch_bounds__(kT, 1) k_cg2d_res(const Res32Args A) {
   constexpr int kWarps = kT / 32, kHalo = 1024 / kT;   // halo nodes per thread
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ float wsum[kWarps], wsum2[kWarps];
+  __shared__ float wsum[kWarps], wsum2[kWarps];   // FP32 per warp
   __shared__ unsigned wmax[kWarps];
   __shared__ int ktab[kTab];
   __shared__ Scalars sc;
@@ -232,6 +232,9 @@ __global__ void __launch_bounds__(kT, 1) k_cg2d_res(const Res32Args A) {
       *reinterpret_cast<float4 *>(SG + o) = ld4(A.s32 + gi);
     }
   }
+  // 2 beta <p, A p_old> from one launch of an inner solve to the next, beside
+  // the arrivals
+  float *carry = reinterpret_cast<float *>(A.msg + 1);
   const bool withhold = st->withhold != 0 && st->iter == 0 && b == 0;
   if (tid == 0) {
     rec.gm = st->gam_m;
@@ -241,7 +244,7 @@ __global__ void __launch_bounds__(kT, 1) k_cg2d_res(const Res32Args A) {
     rec.dF = 0;
     rec.beta = (float)st->beta;
     rec.alpha = 0.f;
-    rec.conj2 = st->conj2;
+    rec.conj2 = (rec.iter == 0) ? 0.f : *carry;
     sc.beta = rec.beta;
     sc.scale = p2f(-st->dF);
     sc.fd = rec.gs - 2 * rec.F;
@@ -292,9 +295,9 @@ __global__ void __launch_bounds__(kT, 1) k_cg2d_res(const Res32Args A) {
       s[i] = fmaf(-sv[i], fmaf(hy, xv[i], yv), pv[i]);
     }
   };
-  // sum over the block of a per-thread FP32 value (FP64 across warps, fixed
-  // order) in warp 0, of a second one in FP32, and the largest of a
-  // non-negative value's bits
+  // sums over the block of two per-thread FP32 values (the first in FP64 across
+  // warps, both in a fixed order) in warp 0, and the largest of a non-negative
+  // value's bits
   auto block_sum = [&](float v, float v2, unsigned mx, int flag, int *any, unsigned *mo,
                        float *s2) {
     for (int o = 16; o > 0; o >>= 1) {
@@ -311,10 +314,12 @@ __global__ void __launch_bounds__(kT, 1) k_cg2d_res(const Res32Args A) {
     double s = 0.0;
     if (wi == 0) {
       s = (lane < kWarps) ? (double)wsum[lane] : 0.0;
-      for (int o = kWarps / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      *mo = __reduce_max_sync(0xffffffffu, lane < kWarps ? wmax[lane] : 0u);
       float t = (lane < kWarps) ? wsum2[lane] : 0.f;
-      for (int o = kWarps / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      for (int o = kWarps / 2; o > 0; o >>= 1) {
+        s += __shfl_xor_sync(0xffffffffu, s, o);
+        t += __shfl_xor_sync(0xffffffffu, t, o);
+      }
+      *mo = __reduce_max_sync(0xffffffffu, lane < kWarps ? wmax[lane] : 0u);
       *s2 = t;
     }
     return s;
@@ -520,11 +525,11 @@ __global__ void __launch_bounds__(kT, 1) k_cg2d_res(const Res32Args A) {
       if (step == 0) {
         sum = block_sum(gam, rs, (unsigned)__float_as_int(rmax), bad, &any, &mo, &rs_b);
         if (tid == 0) {
-          // the second value: largest |r|; <r_new, A p> to 14 bits, the
-          // exponent of the largest |p|, the test's flag
+          // besides <r, r>: <r_new, A p>; and largest |r|, the exponent of the
+          // largest |p|, the test's flag in one word
           sync_put(A.msg, tag, 1, b,
-                   __hiloint2double((int)mo, (int)(((unsigned)__float_as_int(rs_b) & ~0x1ffu) |
-                                                   (pm >> 23) << 1 | (any ? 1u : 0u))));
+                   __hiloint2double((int)mo, (int)((pm >> 23) << 1 | (any ? 1u : 0u))));
+          sync_put(A.msg, tag, 2, b, __hiloint2double(0, __float_as_int(rs_b)));
           sync_put(A.msg, tag, 0, b, sum);
           sync_arrive(A.msg);
         }
@@ -540,8 +545,9 @@ __global__ void __launch_bounds__(kT, 1) k_cg2d_res(const Res32Args A) {
       if (tid == 0) rec.inv_gm = 1.0 / rec.gm;
       arrivals += nblk;
       const bool ok = sync_wait(A.msg, arrivals);
-      double v[kSyncBlocks / 32];
+      double v[kSyncBlocks / 32], v2[kSyncBlocks / 32];
       sync_get(A.msg, tag, 1, nblk, v);
+      sync_get(A.msg, tag, 2, nblk, v2);
       unsigned rm = 0, pmx = 0, fl = 0;
       float rst = 0.f;
 #pragma unroll
@@ -550,7 +556,7 @@ __global__ void __launch_bounds__(kT, 1) k_cg2d_res(const Res32Args A) {
         rm = max(rm, (unsigned)__double2hiint(v[j]));
         pmx = max(pmx, (lo >> 1) & 0xffu);
         fl |= lo & 1u;
-        rst += __int_as_float((int)(lo & ~0x1ffu));
+        rst += __int_as_float(__double2loint(v2[j]));
       }
       sync_get(A.msg, tag, 0, nblk, v);
       const double G = sync_sum(v);
@@ -628,7 +634,7 @@ __global__ void __launch_bounds__(kT, 1) k_cg2d_res(const Res32Args A) {
       st->fd = rec.gs - 2 * rec.F;
       st->total_iter += rec.iter - st->iter;
       st->iter = rec.iter;
-      st->conj2 = rec.conj2;
+      *carry = rec.conj2;
       if (stop != 0) {
         if (stop == kStall) st->stalled = 1;
         atomicCAS(&st->status, (int)EIK_OK, stop == kStall ? (int)EIK_OK : stop - kStop);
