@@ -39,6 +39,7 @@
 #include "eik_launch.h"
 #include "eik_mg.h"
 #include "eik_mixed.h"
+#include "eik_pair3d.h"
 #include "eik_res32.h"
 
 namespace eik {
@@ -473,6 +474,11 @@ struct MixedState {
   MgState *mg = nullptr;
   // resident inner CG (2D grids that fit on chip, no explicit kernel variant)
   Res32Plan res;
+  // two-pass inner CG (3D grids, no explicit kernel variant)
+  Pair3Plan pair;
+  // which of them the current refinement uses (pick_kernels)
+  bool use_res = false, use_pair = false;
+  bool graph_pair = false;   // the graph holds two-pass iterations
   cudaGraphExec_t graph = nullptr;
   int64_t launches[8] = {0};
   // per-launch CUDA-event timing of the inner passes when profiling
@@ -626,8 +632,10 @@ eik_status mixed_create(MixedState **out, const Grid &g, const TileCount &tc, in
     g_msg = "cannot reserve shared memory for the coarse estimate";
     return EIK_ERR_CUDA;
   }
-  if (precond == EIK_PRECOND_JACOBI && tile_override == 0)
+  if (precond == EIK_PRECOND_JACOBI && tile_override == 0) {
     res32_plan(&m->res, g, m->cg, num_sms, s);
+    pair3_plan(&m->pair, g, m->cg, num_sms, s);
+  }
   if (precond == EIK_PRECOND_MULTIGRID) {
     const eik_status ms = mg_create(&m->mg, g, m->cg, m->px, num_sms, s);
     if (ms != EIK_OK) {
@@ -684,6 +692,7 @@ void mixed_destroy(MixedState *m) {
   if (!m) return;
   if (m->mg) mg_destroy(m->mg);
   res32_destroy(&m->res);
+  pair3_destroy(&m->pair);
   if (m->graph) cudaGraphExecDestroy(m->graph);
   for (auto &e : m->ev)
     if (e) cudaEventDestroy(e);
@@ -711,11 +720,20 @@ static void launch_residual(MixedState *m, const MixedArgs &a) {
   m->launches[2]++;
 }
 
+// One inner iteration as one or two launches: reads direction set `set`.
+static void inner_iter(MixedState *m, int set, cudaStream_t s) {
+  if (m->use_pair) pair3_iter(m->pair, m->g, m->cg, m->bufs, set, s);
+  else cg32_iter(m->plan, m->g, m->cg, m->bufs, set, s);
+}
+
 static eik_status build_graph(MixedState *m, cudaStream_t s) {
-  if (m->graph) return EIK_OK;
+  if (m->graph && m->graph_pair == m->use_pair) return EIK_OK;
+  if (m->graph) MCK(cudaGraphExecDestroy(m->graph));
+  m->graph = nullptr;
+  m->graph_pair = m->use_pair;
   cudaGraph_t graph;
   MCK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-  for (int k = 0; k < kInnerGraphIters; ++k) cg32_iter(m->plan, m->g, m->cg, m->bufs, k & 1, s);
+  for (int k = 0; k < kInnerGraphIters; ++k) inner_iter(m, k & 1, s);
   MCK(cudaStreamEndCapture(s, &graph));
   MCK(cudaGraphInstantiate(&m->graph, graph, 0));
   MCK(cudaGraphDestroy(graph));
@@ -794,9 +812,9 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
     st.alpha = 0.0;
     st.beta = 0.0;
     st.F = 0;
-    // (the resident kernel moves r to its frame first; the one-pass kernels do
-    // so from their first pass's maximum)
-    st.dF = m->res.ok ? std::max(-126, std::min(126, std::ilogb(st.r_inf))) : 0;
+    // (the resident and the two-pass kernels move r to its frame first; the
+    // one-pass kernels do so from their first pass's maximum)
+    st.dF = (m->use_res || m->use_pair) ? std::max(-126, std::min(126, std::ilogb(st.r_inf))) : 0;
     st.fd = st.rho_s;
     st.iter = 0;
     st.done = 0;
@@ -807,7 +825,13 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
     st.withhold = (a.opt.test_flags & 1) ? 1 : 0;
     st.mode = (outer == 0 || !std::isfinite(cw) || careful) ? 0 : 1;
     st.thresh = (float)(red * st.r_inf);
-    st.theta = (float)std::max(0.5 * tol, 1e-3 * cw);
+    // a step whose aim is below tol is probably the last one: the two-sum
+    // kernels then go to tol / 8 (on eight grids at tol 1e-6 and 1e-8: 2 % more
+    // iterations, S up to 12 times nearer; at tol / 2 a 2048^2 solve to 1e-6
+    // ended at cw = 9.6e-7 with S off by 1.1e-6, at tol / 8 by 1.5e-7)
+    const double aim = 1e-3 * cw;
+    st.theta = (float)(aim < tol && (m->use_res || m->use_pair) ? 0.125 * tol
+                                                              : std::max(0.5 * tol, aim));
     if (m->batch) {
       // the batch's passes make the first pass of this solve w = A r
       st.seq = batch_exec_ticket(m->batch, m->bidx);
@@ -837,12 +861,15 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
       if (m->profile && !m->ev[0])
         for (auto &e : m->ev) MCK(cudaEventCreate(&e));
       if (m->profile) MCK(cudaEventRecord(m->ev[0], s));
-      // (the resident kernel starts from the residual's <r, r>; it has no
-      // initial pass of its own, and the count below is of inner solves)
-      if (!m->res.ok) cg32_init(m->plan, g, m->cg, m->bufs, 0, s);
+      // (the resident and the two-pass kernels start from the residual's
+      // <r, r>; they have no initial pass, and the count below is of inner
+      // solves)
+      const bool init = !m->use_res && !m->use_pair;
+      const int per_iter = m->use_pair ? 2 : 1;   // launches
+      if (init) cg32_init(m->plan, g, m->cg, m->bufs, 0, s);
       m->launches[3]++;
       MCK(cudaGetLastError());
-      if (m->profile && !m->res.ok) {
+      if (m->profile && init) {
         MCK(cudaEventRecord(m->ev[1], s));
         MCK(cudaStreamSynchronize(s));
         float t = 0.f;
@@ -852,14 +879,14 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
       }
       int before = 0;
       for (int it = 0;; ++it) {
-        if (m->res.ok) {
+        if (m->use_res) {
           if (m->profile) MCK(cudaEventRecord(m->ev[1], s));
           const cudaError_t e = launch_res32(&m->res, g, m->cg, m->bufs, s);
           if (e == cudaErrorCooperativeLaunchTooLarge) {
             // fewer SMs than the device reports (a partitioned context): the
             // one-pass kernels from here on; nothing has run yet
             cudaGetLastError();
-            m->res.ok = false;
+            m->res.ok = m->use_res = false;
             const eik_status gs = build_graph(m, s);
             if (gs != EIK_OK) return gs;
             cg32_init(m->plan, g, m->cg, m->bufs, 0, s);
@@ -872,12 +899,12 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
         } else if (m->profile) {
           // one timed iteration per host check: no launch runs past convergence
           MCK(cudaEventRecord(m->ev[1], s));
-          cg32_iter(m->plan, g, m->cg, m->bufs, it & 1, s);
+          inner_iter(m, it & 1, s);
           MCK(cudaEventRecord(m->ev[2], s));
-          m->launches[4] += 1;
+          m->launches[4] += per_iter;
         } else {
           MCK(cudaGraphLaunch(m->graph, s));
-          m->launches[4] += kInnerGraphIters;
+          m->launches[4] += (int64_t)kInnerGraphIters * per_iter;
         }
         MCK(cudaMemcpyAsync(m->h_st, m->st, sizeof(MixCtl), cudaMemcpyDeviceToHost, s));
         MCK(cudaStreamSynchronize(s));
@@ -887,7 +914,7 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
           float t = 0.f;
           MCK(cudaEventElapsedTime(&t, m->ev[1], m->ev[2]));
           m->ms[4] += t;
-          m->timed[4] += m->res.ok ? done_now : 1;   // times are per iteration
+          m->timed[4] += m->use_res ? done_now : 1;   // times are per iteration
         }
         if (m->h_st->done) break;
       }
@@ -943,17 +970,12 @@ eik_status mixed_solve(MixedState *m, const MixedArgs &a, int *inner_iters, int 
   m->launches[0] += 3;
   m->launches[1] += 1;
   MCK(cudaGetLastError());
-  if (!m->batch && !m->mg && !m->res.ok) {
-    eik_status gs = build_graph(m, s);
-    if (gs != EIK_OK) return gs;
-  }
-
   // multigrid inner solves take wider bands: one global refinement holds
   // ranges up to kMgSweepBits (its inner products lose the far field only
   // where their weights 2^(-2 kx) leave the FP64 range)
   const int band_bits = (a.opt.band_bits > 0) ? a.opt.band_bits : (m->mg ? kMgBandBits : kBandBits);
   int kmin = 0, kmax = 0;
-  if (a.opt.band_bits >= 0 || m->mg) {
+  if (a.opt.band_bits >= 0 || m->mg || m->res.ok || m->pair.ok) {
     std::vector<int> hk(m->cg.ncell);
     MCK(cudaMemcpyAsync(hk.data(), m->kx, sizeof(int) * hk.size(), cudaMemcpyDeviceToHost, s));
     MCK(cudaStreamSynchronize(s));
@@ -968,13 +990,27 @@ eik_status mixed_solve(MixedState *m, const MixedArgs &a, int *inner_iters, int 
     if (ms != EIK_OK) g_msg = mg_last_error();
     return ms;
   };
+  // Inner-CG kernels for a refinement over `span` powers of two of kx.  The
+  // two-sum kernels take those up to kSweepBits, which is every one unless the
+  // sweeps are switched off or their bands widened: past that range the FP32
+  // directions lose conjugacy early, and the one-pass recurrence recovers
+  // where the two-sum one may not (512^2, hbar = 2.6 h, no sweeps: its
+  // residual grew from step to step).  The test hook withholds a copy of the
+  // one-pass kernels in 3D.
+  auto pick_kernels = [&](int span) -> eik_status {
+    if (m->batch || m->mg) return EIK_OK;
+    m->use_res = m->res.ok && span <= kSweepBits;
+    m->use_pair = m->pair.ok && span <= kSweepBits && !(a.opt.test_flags & 1);
+    return m->use_res ? EIK_OK : build_graph(m, s);
+  };
   const int max_outer = (a.opt.max_outer > 0) ? a.opt.max_outer : 30;
   int total = 0, outer = 0;
   eik_status result;
   const int sweep_bits = (a.opt.band_bits > 0) ? 2 * a.opt.band_bits
                                                : (m->mg ? kMgSweepBits : kSweepBits);
   if (a.opt.band_bits < 0 || kmax - kmin <= sweep_bits) {
-    const eik_status ms = mg_rebuild(kmin);
+    eik_status ms = mg_rebuild(kmin);
+    if (ms == EIK_OK) ms = pick_kernels(kmax - kmin);
     if (ms != EIK_OK) return ms;
     result = refine(m, a, INT_MIN, INT_MAX, max_outer, &total, &outer, res_cw, trace);
   } else {
@@ -994,7 +1030,8 @@ eik_status mixed_solve(MixedState *m, const MixedArgs &a, int *inner_iters, int 
                                                       m->s32);
         m->launches[0]++;
         MCK(cudaGetLastError());
-        const eik_status ms = mg_rebuild(lo);
+        eik_status ms = mg_rebuild(lo);
+        if (ms == EIK_OK) ms = pick_kernels(hi - lo);
         if (ms != EIK_OK) return ms;
         if (trace) fprintf(stderr, "[mixed] sweep %d band [%d, %d)\n", sweep, lo, hi);
         const eik_status bs = refine(m, a, lo, hi, max_outer, &total, &outer, res_cw, trace);
@@ -1012,6 +1049,8 @@ eik_status mixed_solve(MixedState *m, const MixedArgs &a, int *inner_iters, int 
     if (result == EIK_ERR_NOT_CONVERGED && kmax - kmin <= kGlobalFinishBits &&
         total < a.opt.max_iter) {
       // a moderate range: finish with refinement steps over the whole grid
+      const eik_status ms = pick_kernels(kmax - kmin);
+      if (ms != EIK_OK) return ms;
       result = refine(m, a, INT_MIN, INT_MAX, max_outer, &total, &outer, res_cw, trace);
     }
     if (result == EIK_ERR_NOT_CONVERGED) g_msg = "level-set sweeps did not converge";
