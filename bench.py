@@ -45,6 +45,8 @@ ALGO_BYTES_PER_NODE = {
     # one single-reduction FP32 inner iteration: read r, p, sig, d; write r,
     # p (other buffer set) and d (7 x 4 B); the checking passes (every 4th
     # in later refinement steps) also read the FP32 iterate, not counted
+    # (the two-pass 3D kernels move 11 words, the resident 2D ones d at most;
+    # their times are per iteration, and the same 7 words are counted)
     "mixed_cg": 28,
     "mixed_cg_init": 8,  # first pass of an inner solve: read r, sig
     # FP64 residual of a refinement step: read sig, x (f64); write r, p, d,
@@ -853,9 +855,12 @@ def roofline(res, inst, wname, only=None):
                 "share_of_kernel_time": round(cand[dom][2] / total, 3) if total else None}
     algo = algo_bytes(dom, inst) * inst.n
     achieved = algo / (avg_ms * 1e-3) / 1e9
+    # the recorded inner-CG counters are the one-pass kernels', which have a
+    # first pass of their own (the resident and the two-pass kernels have none)
+    traffic = (ncu_traffic(dom, wname) if dom != "mixed_cg" or "mixed_cg_init" in km else None)
     return {"bound": "hbm", "kernel": dom, "achieved": round(achieved, 1),
             "peak": peak, "peak_source": peak_src, "unit": "GB/s",
-            "frac": round(achieved / peak, 4), "traffic": ncu_traffic(dom, wname),
+            "frac": round(achieved / peak, 4), "traffic": traffic,
             "algorithmic_bytes_per_launch": algo, "avg_launch_ms": avg_ms,
             "share_of_kernel_time": round(cand[dom][2] / total, 3) if total else None}
 

@@ -27,10 +27,9 @@
 
 namespace eik {
 
-// Recurrence between the two passes: <r,r> =
-// gm 2^gs with gm in [0.5, 1), frame F of the stored r, factor `scale` that
-// moves them there, <p, A p> and 2 beta <p, A p_old> of the next direction
-// (units of 2^gs).
+// Recurrence between the two passes: <r,r> = gm 2^gs with gm in [0.5, 1), frame
+// F that r and p are in once multiplied by `scale` (dir does so for p, step for
+// r), <p, A p> and 2 beta <p, A p_old> of the next direction (units of 2^gs).
 struct PairCtl {
   double gm;
   int gs, F, fd, check;

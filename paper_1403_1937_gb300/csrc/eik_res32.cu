@@ -14,13 +14,14 @@
 // redundant halo arithmetic and no second stencil on r.  s = A p is computed
 // once for <p,s> and again for r, since holding it would take another quarter
 // of the registers.
-// Measured per iteration (one-pass kernel, this one): 611 x 733 26 us, 12 us;
-// 512^2 23 us, 9 us; 2048^2 45 us, 37 us (there 128 registers a thread are not
+// Measured per iteration (one-pass kernel, this one): 611 x 733 26 us, 9.8 us;
+// 512^2 23 us, 9 us; 2048^2 45 us, 33 us (there 128 registers a thread are not
 // enough for 64 values of r, and the spills bound it).
 //
-// Split: tiles of up to 128 columns (a lane owns four of them) and 256 rows, at most one block per SM, and no more blocks than keep kMinNodes
-// nodes each: the two sums take about 4 us whatever the tile, so smaller ones
-// do not pay, and the SMs left free run other solves.  Sums are FP32 per
+// Split: tiles of up to 128 columns (a lane owns four of them) and 256 rows, at
+// most one block per SM, and no more blocks than keep kMinNodes nodes each: the
+// two sums take about 4 us whatever the tile, so smaller ones do not pay, and
+// the SMs left free run other solves.  Sums are FP32 per
 // warp, FP64 across warps and blocks in a fixed order: deterministic, and the
 // split depends on the grid alone.
 #include <math.h>
