@@ -412,7 +412,10 @@ __global__ void __launch_bounds__(kT, 1) k_cg64_res(const Res64Args A) {
       sync_get(A.msg, tag, 0, nblk, v);
       const double rr = sync_sum(v);
       if (tid == 0) {
-        sh_val = rr * inv_rho;
+        // (below about 5.6e-309 rho has no finite reciprocal; a solve whose phi
+        // spans more than 1e150 passes through there before rho reaches 0 and
+        // the loop ends for a restart from the true residual)
+        sh_val = finite64(inv_rho) ? rr * inv_rho : rr / rho;
         const bool conv = cw ? (check && !fl) : rr <= nw;
         sh_stop = !ok ? kLate
                   : !finite64(rr) ? kStop + EIK_ERR_BREAKDOWN
