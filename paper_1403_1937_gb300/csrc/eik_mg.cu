@@ -65,13 +65,19 @@ constexpr float kOmega = 8.0f / 9.0f;   // Chebyshev-optimal single step on [1/4
 constexpr int kGraphIters = 2;          // even: the direction buffers alternate
 // an inner solve that has not met its test after this many iterations ends
 // (the refinement step then judges progress from the true residual)
-constexpr int kMaxInnerIters = 300;
-// and so does one whose largest residual grows by this factor: the FP32
-// recurrence has come apart, and every power of ten costs a refinement step
-// to take back (measured: a 400^2 solve with hbar = 2 h whose residual had
-// grown by 1e14 and 1e18 took 18 steps, or all 30, to return).  Its correction
-// is dropped (MixCtl.stalled = 2).
+constexpr int kMaxInnerIters = 1000;
+// An inner solve is cut off (MixCtl.stalled = 2) where its largest residual has
+// grown by kMaxGrowth, or has not fallen below its smallest value for kMaxIdle
+// iterations: the FP32 recurrence has come apart, and every power of ten that
+// the residual has grown by costs a refinement step to take back (measured
+// without the cut-off: a 400^2 solve with hbar = 2 h whose residual had grown by
+// 1e14 and 1e18 took 18 steps, or all 30, to return).  Its correction is dropped
+// and the same solve, which is deterministic, runs again up to the iteration
+// with the smallest residual.  Where that was not below half of the first one,
+// growth may be what the solve needs (the maximum norm in kx units does not
+// fall steadily in CG), and it runs again without a cut-off.
 constexpr float kMaxGrowth = 1e4f;
+constexpr int kMaxIdle = 200;
 thread_local std::string g_msg = "no error";
 
 enum { kW = 0, kE = 1, kS = 2, kN = 3, kB = 4, kT = 5, kDirs = 6 };
@@ -92,7 +98,10 @@ struct MgCtl {
   double alpha, beta;
   int iter, max_iter, done, status, stalled, mode, first, kmin;
   float thresh, theta;
-  float r_limit;     // the inner solve ends where max |r| grows past this
+  float r_limit;     // the inner solve is cut off where max |r| grows past this,
+  int max_idle;      // or after this many iterations without a new smallest one
+  float r_best;      // smallest max |r| so far and its iteration (0: the start)
+  int best_iter;
   unsigned int counter[4];
 };
 
@@ -995,13 +1004,19 @@ k_mg_step(int64_t n4, const float4 *__restrict__ p, const float4 *__restrict__ q
     ctl->counter[2] = 0u;
     ctl->iter += 1;
     const bool conv = (mode == 0) ? (rm <= ctl->thresh) : (vi == 0);
+    if (rm < ctl->r_best) {
+      ctl->r_best = rm;
+      ctl->best_iter = ctl->iter;
+    }
     if (!isfinite(rm)) {
       ctl->status = EIK_ERR_BREAKDOWN;
       ctl->done = 1;
-    } else if (conv || ctl->iter >= ctl->max_iter) {
+    } else if (conv) {
       ctl->done = 1;
-    } else if (rm > ctl->r_limit) {
+    } else if (rm > ctl->r_limit || ctl->iter - ctl->best_iter >= ctl->max_idle) {
       ctl->stalled = 2;
+      ctl->done = 1;
+    } else if (ctl->iter >= ctl->max_iter) {
       ctl->done = 1;
     }
   }
@@ -1261,7 +1276,7 @@ static void launch_iter(MgState *mg, const MgFine &f, int set, cudaStream_t s) {
 
 static int launches_per_iter(const MgState *mg) { return 2 * (tail_start(mg) - 1) + 5; }
 
-eik_status mg_inner(MgState *mg, const MgFine &f, MixCtl *h_st, cudaStream_t s) {
+eik_status mg_inner(MgState *mg, const MgFine &f, MixCtl *h_st, int *again, cudaStream_t s) {
   if (mg->graph && (f.r != mg->bound.r || f.d != mg->bound.d || f.xref != mg->bound.xref ||
                     f.s32 != mg->bound.s32 || f.kx != mg->bound.kx)) {
     cudaGraphExecDestroy(mg->graph);
@@ -1278,11 +1293,14 @@ eik_status mg_inner(MgState *mg, const MgFine &f, MixCtl *h_st, cudaStream_t s) 
   }
   MgCtl c{};
   c.kmin = mg->h_ctl->kmin;
-  c.max_iter = std::max(1, std::min(h_st->max_iter, kMaxInnerIters));
+  const bool guard = *again == kMgFirst;
+  c.max_iter = std::max(1, std::min(h_st->max_iter, *again > 0 ? *again : kMaxInnerIters));
   c.mode = h_st->mode;
   c.thresh = h_st->thresh;
   c.theta = h_st->theta;
-  c.r_limit = kMaxGrowth * (float)h_st->r_inf;
+  c.r_best = (float)h_st->r_inf;
+  c.r_limit = guard ? kMaxGrowth * c.r_best : INFINITY;
+  c.max_idle = guard ? kMaxIdle : INT_MAX;
   c.first = 1;
   *mg->h_ctl = c;
   GCK(cudaMemcpyAsync(mg->ctl, mg->h_ctl, sizeof(MgCtl), cudaMemcpyHostToDevice, s));
@@ -1311,6 +1329,9 @@ eik_status mg_inner(MgState *mg, const MgFine &f, MixCtl *h_st, cudaStream_t s) 
   h_st->status = mg->h_ctl->status;
   h_st->stalled = mg->h_ctl->stalled;
   h_st->done = 1;
+  *again = kMgFirst;
+  if (h_st->stalled == 2)
+    *again = (mg->h_ctl->r_best <= 0.5f * c.r_best) ? mg->h_ctl->best_iter : kMgNoCutoff;
   return EIK_OK;
 }
 

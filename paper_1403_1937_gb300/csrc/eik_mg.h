@@ -24,9 +24,13 @@ eik_status mg_create(MgState **out, const Grid &g, const CellGrid &cg, int px, i
 // every coarser level.  kmin = smallest cell exponent (reference of the
 // inner-product weights).
 eik_status mg_setup(MgState *mg, const MgFine &f, int kmin, cudaStream_t s);
-// One inner solve of a refinement step.  Reads mode, thresh, theta and
+// One inner solve of a refinement step.  Reads mode, thresh, theta, r_inf and
 // max_iter from *h_st and returns iter, status, stalled and done there.
-eik_status mg_inner(MgState *mg, const MgFine &f, MixCtl *h_st, cudaStream_t s);
+// *again: kMgFirst; after a solve that was cut off (stalled = 2, its correction
+// is to be dropped) it holds how the same solve is to run again, from the same
+// residual: up to that many iterations, or without a cut-off.
+constexpr int kMgFirst = -1, kMgNoCutoff = 0;
+eik_status mg_inner(MgState *mg, const MgFine &f, MixCtl *h_st, int *again, cudaStream_t s);
 void mg_destroy(MgState *mg);
 int mg_levels(const MgState *mg);
 int64_t mg_launches(const MgState *mg);

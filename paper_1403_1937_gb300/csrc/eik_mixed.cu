@@ -758,9 +758,9 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
   int total = *total_io, outer = 0;
   double best_cw = INFINITY, last_cw = INFINITY;
   int stall = 0;
-  // set once an inner solve has come apart: the later ones aim at the smaller
-  // reduction of the first step, which they reach before they do
-  bool careful = false;
+  // how the next multigrid inner solve runs: other than kMgFirst after one that
+  // was cut off, whose correction was dropped (mg_inner)
+  int again = kMgFirst;
   eik_status result = EIK_ERR_NOT_CONVERGED;
   for (;;) {
     MixCtl init{};
@@ -799,7 +799,7 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
     if (!std::isfinite(cw) || cw < 0.5 * best_cw) {
       if (std::isfinite(cw)) best_cw = cw;
       stall = 0;
-    } else if (!recovering && ++stall >= 2) {
+    } else if (again == kMgFirst && !recovering && ++stall >= 2) {
       g_msg = "mixed refinement stopped making progress";
       break;
     }
@@ -823,7 +823,7 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
     st.fault = 0;
     st.max_iter = std::max(1, a.opt.max_iter - total);
     st.withhold = (a.opt.test_flags & 1) ? 1 : 0;
-    st.mode = (outer == 0 || !std::isfinite(cw) || careful) ? 0 : 1;
+    st.mode = (outer == 0 || !std::isfinite(cw)) ? 0 : 1;
     st.thresh = (float)(red * st.r_inf);
     // a step whose aim is below tol is probably the last one: the two-sum
     // kernels then go to tol / 8 (on eight grids at tol 1e-6 and 1e-8: 2 % more
@@ -841,7 +841,7 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
     MCK(cudaMemcpyAsync(m->st, m->h_st, sizeof(MixCtl), cudaMemcpyHostToDevice, s));
     if (m->mg) {
       const MgFine fine{m->r32[0], m->d32, m->xref, m->s32, m->kx, m->St};
-      const eik_status ms = mg_inner(m->mg, fine, m->h_st, s);
+      const eik_status ms = mg_inner(m->mg, fine, m->h_st, &again, s);
       if (ms != EIK_OK) {
         g_msg = mg_last_error();
         result = ms;
@@ -920,7 +920,7 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
       }
     }
     total += m->h_st->iter;
-    ++outer;
+    if (again == kMgFirst) ++outer;
     if (trace)
       fprintf(stderr,
               "[mixed]   inner end: iters %d status %d stalled %d alpha %.3e beta %.3e F %d\n",
@@ -936,10 +936,7 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
       result = EIK_ERR_BREAKDOWN;
       break;
     }
-    if (m->h_st->stalled == 2 && !careful) {
-      careful = true;   // the correction is dropped
-      continue;
-    }
+    if (again != kMgFirst) continue;   // the correction is dropped
     k_mixed_update<<<blocks(g.n), kThreads, 0, s>>>(g.n, g.nx, m->px, m->d32, m->x64);
     m->launches[5]++;
     MCK(cudaGetLastError());
