@@ -111,6 +111,9 @@ __device__ __forceinline__ bool sync_wait(unsigned long long *msg, unsigned targ
       }
     }
   }
+  // (the shuffle orders no memory accesses: the other lanes' reads of the
+  // partials come after lane 0's acquire by this barrier)
+  __syncwarp();
   return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 // Warp 0, after sync_wait: partial v of the blocks lane, lane + 32, ... (0 past
