@@ -31,9 +31,9 @@ namespace eik {
 // F that r and p are in once multiplied by `scale` (dir does so for p, step for
 // r), <p, A p> and 2 beta <p, A p_old> of the next direction (units of 2^gs).
 struct PairCtl {
-  double gm;
+  double gm, beta, ps, conj2;
   int gs, F, fd, check;
-  float alpha, alphaF, beta, scale, thetaF, ps, conj2;
+  float alpha, alphaF, scale, thetaF;
   unsigned pexp;          // exponent bits of the largest |p|
   unsigned counter[2];
 };
@@ -119,7 +119,7 @@ k_pair_dir(const PairArgs A, int tiles_x, int tiles_y, int zc, int ntiles) {
   const bool start = st->iter == 0;
   const int dF0 = st->dF, F0 = st->F + dF0;
   const float scale = start ? p2f(-dF0) : c->scale;
-  const float beta = start ? 0.f : c->beta * scale;
+  const float beta = start ? 0.f : (float)c->beta * scale;
   const int fd = start ? st->gam_s - 2 * F0 : c->fd;
   const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
   const int mask = A.cg.B - 1, lg = A.cg.lgB, layer = A.cg.cx * A.cg.cy;
@@ -333,7 +333,7 @@ k_pair_dir(const PairArgs A, int tiles_x, int tiles_y, int zc, int ntiles) {
     c->F = F0;
     c->fd = fd;
     c->scale = scale;
-    c->conj2 = 0.f;
+    c->conj2 = 0.0;
     c->check = 0;
     c->thetaF = ldexpf(st->theta, -F0);
   }
@@ -342,10 +342,10 @@ k_pair_dir(const PairArgs A, int tiles_x, int tiles_y, int zc, int ntiles) {
   // unnoticed; once the difference is not positive the inner solve ends, its
   // correction so far is kept, and the refinement restarts from the true
   // residual (the resident 2D kernel does the same)
-  const double gm = c->gm, den = ps - (double)c->conj2;
+  const double gm = c->gm, den = ps - c->conj2;
   const bool pos = ps > 0.0 && den > 0.0 && isfinite(den);
   const float al = pos ? (float)(gm / den) : 0.f;
-  c->ps = (float)ps;
+  c->ps = ps;
   c->alpha = al;
   c->alphaF = ldexpf(al, c->F);
   if (gm == 0.0) finish(st, EIK_OK, false);
@@ -413,7 +413,7 @@ k_pair_step(const PairArgs A, int bx, int by) {
   }
   if (!last_block(&c->counter[1], &flag)) return;
   const double G = sum_partials(part, gridDim.x, shd);
-  const float rst = (float)sum_partials(part + gridDim.x, gridDim.x, shd);
+  const double rst = sum_partials(part + gridDim.x, gridDim.x, shd);
   unsigned m = 0, fl = 0;
   for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
     const uint2 v = __ldcg(mx + b);
@@ -440,8 +440,8 @@ k_pair_step(const PairArgs A, int bx, int by) {
     // 2 beta <p, A p_old> = 2 beta (<r_new, A p> + beta <p, A p>)
     int eg;
     const double gn = frexp(G, &eg);
-    const float be = ldexpf((float)(gn / c->gm), eg);
-    c->conj2 = ldexpf(2.f * be * fmaf(be, c->ps, rst), -eg);
+    const double bm = gn / c->gm, be = scalbn(bm, eg);
+    c->conj2 = 2.0 * bm * fma(be, c->ps, rst);
     c->beta = be;
     c->gm = gn;
     c->gs += eg;

@@ -14,16 +14,22 @@
 // redundant halo arithmetic and no second stencil on r.  s = A p is computed
 // once for <p,s> and again for r, since holding it would take another quarter
 // of the registers.
-// Measured per iteration (one-pass kernel, this one): 611 x 733 26 us, 9.8 us;
-// 512^2 23 us, 9 us; 2048^2 45 us, 33 us (there 128 registers a thread are not
-// enough for 64 values of r, and the spills bound it).
+// Measured per iteration of a solve (one-pass kernel, this one): 300 x 260
+// 25.9 us, 10.5 us; 512^2 25.6 us, 8.6 us; 611 x 733 25.7 us, 10.1 us; 1500^2
+// 33.0 us, 18.4 us; 2048^2 46.1 us, 34.4 us.  128 registers a thread are not
+// enough beside r: tiles of up to 32 rows spill nothing, of 64 rows 72 B, of 128
+// 268 B, of 256 592 B a thread (bytes stored), which bounds the largest grids.
+// <r_new, A p>, <p, A p> and beta take FP64 like <r, r>, as in the one-pass
+// kernels; adding <r_new, A p> in a second warp keeps that off the chain that
+// the block waits for (in the same warp: 0.3 us an iteration).
 //
-// Split: tiles of up to 128 columns (a lane owns four of them) and 256 rows, at
-// most one block per SM, and no more blocks than keep kMinNodes nodes each: the
-// two sums take about 4 us whatever the tile, so smaller ones do not pay, and
-// the SMs left free run other solves.  Sums are FP32 per
-// warp, FP64 across warps and blocks in a fixed order: deterministic, and the
-// split depends on the grid alone.
+// Split: tiles of up to 128 columns (a lane owns four of them) and 256 rows
+// (222 KB of p and sigma), at most one block per SM: with 152 SMs 2048 x 2048 is
+// the largest square, and larger grids take the one-pass kernels.  There are
+// no more blocks than keep kMinNodes nodes each: the two sums take about 4 us
+// whatever the tile, so smaller ones do not pay, and the SMs left free run
+// other solves.  Sums are FP32 per warp, FP64 across warps and blocks in a fixed
+// order: deterministic, and the split depends on the grid alone.
 #include <math.h>
 
 #include <algorithm>
@@ -60,12 +66,13 @@ struct Scalars {
   int fd, check, stop;
 };
 // The recurrence itself, kept by thread 0: <r,r> = gm 2^gs with gm in
-// [0.5, 1), frame F (and the step dF to it that r and p still lack), <p, A p>
-// and 2 beta <p, A p_old> of the next direction (units of 2^gs).
+// [0.5, 1), frame F (and the step dF to it that r and p still lack), beta and its
+// mantissa, <p, A p>, <r_new, A p> and 2 beta <p, A p_old> of the next direction
+// (units of 2^gs).
 struct Recurrence {
-  double gm, inv_gm;
+  double gm, inv_gm, beta, bm, ps, rst, conj2;
   int gs, F, dF, iter;
-  float beta, alpha, ps, conj2;
+  float alpha;
 };
 // outcomes besides 0 (go on): kStop + eik_status, kStall (positivity lost), a
 // wait that ran out
@@ -235,7 +242,7 @@ __global__ void __launch_bounds__(kT, 1) k_cg2d_res(const Res32Args A) {
   }
   // 2 beta <p, A p_old> from one launch of an inner solve to the next, beside
   // the arrivals
-  float *carry = reinterpret_cast<float *>(A.msg + 1);
+  double *carry = reinterpret_cast<double *>(A.msg + 1);
   const bool withhold = st->withhold != 0 && st->iter == 0 && b == 0;
   if (tid == 0) {
     rec.gm = st->gam_m;
@@ -243,10 +250,11 @@ __global__ void __launch_bounds__(kT, 1) k_cg2d_res(const Res32Args A) {
     rec.F = st->F + st->dF;
     rec.iter = st->iter;
     rec.dF = 0;
-    rec.beta = (float)st->beta;
+    rec.beta = st->beta;
     rec.alpha = 0.f;
-    rec.conj2 = (rec.iter == 0) ? 0.f : *carry;
-    sc.beta = rec.beta;
+    rec.bm = rec.ps = rec.rst = 0.0;
+    rec.conj2 = (rec.iter == 0) ? 0.0 : *carry;
+    sc.beta = (float)rec.beta;
     sc.scale = p2f(-st->dF);
     sc.fd = rec.gs - 2 * rec.F;
     sc.thetaF = ldexpf(st->theta, -rec.F);
@@ -296,11 +304,13 @@ __global__ void __launch_bounds__(kT, 1) k_cg2d_res(const Res32Args A) {
       s[i] = fmaf(-sv[i], fmaf(hy, xv[i], yv), pv[i]);
     }
   };
-  // sums over the block of two per-thread FP32 values (the first in FP64 across
-  // warps, both in a fixed order) in warp 0, and the largest of a non-negative
-  // value's bits
+  // sums over the block of two per-thread FP32 values, FP64 across warps in a
+  // fixed order: in the lower (v) and the upper (v2) half of warp 0, so that
+  // the second takes no instructions of its own; and the largest of a
+  // non-negative value's bits
+  static_assert(kWarps == 16, "a half warp adds the warps' values");
   auto block_sum = [&](float v, float v2, unsigned mx, int flag, int *any, unsigned *mo,
-                       float *s2) {
+                       double *s2) {
     for (int o = 16; o > 0; o >>= 1) {
       v += __shfl_xor_sync(0xffffffffu, v, o);
       v2 += __shfl_xor_sync(0xffffffffu, v2, o);
@@ -314,14 +324,10 @@ __global__ void __launch_bounds__(kT, 1) k_cg2d_res(const Res32Args A) {
     *any = __syncthreads_or(flag);
     double s = 0.0;
     if (wi == 0) {
-      s = (lane < kWarps) ? (double)wsum[lane] : 0.0;
-      float t = (lane < kWarps) ? wsum2[lane] : 0.f;
-      for (int o = kWarps / 2; o > 0; o >>= 1) {
-        s += __shfl_xor_sync(0xffffffffu, s, o);
-        t += __shfl_xor_sync(0xffffffffu, t, o);
-      }
+      s = (double)(lane < kWarps ? wsum[lane] : wsum2[lane - kWarps]);
+      for (int o = kWarps / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (s2) *s2 = __shfl_sync(0xffffffffu, s, kWarps);
       *mo = __reduce_max_sync(0xffffffffu, lane < kWarps ? wmax[lane] : 0u);
-      *s2 = t;
     }
     return s;
   };
@@ -381,8 +387,8 @@ __global__ void __launch_bounds__(kT, 1) k_cg2d_res(const Res32Args A) {
     }
     int any;
     unsigned mo = 0;
-    float rs_b = 0.f;
-    double sum = block_sum(pap, 0.f, (unsigned)__float_as_int(pmax), late, &any, &mo, &rs_b);
+    double rs_b = 0.0;
+    double sum = block_sum(pap, 0.f, (unsigned)__float_as_int(pmax), late, &any, &mo, nullptr);
     ++tag;
     unsigned pm = mo;
     if (wi == 0) {
@@ -391,6 +397,8 @@ __global__ void __launch_bounds__(kT, 1) k_cg2d_res(const Res32Args A) {
         sync_put(A.msg, tag, 0, b, sum);
         sync_arrive(A.msg);
       }
+      // (while the sums travel) <p, A p_old> = <r_new, A p> + beta <p, A p>
+      if (tid == 0 && it > 0) rec.conj2 = 2.0 * rec.bm * fma(rec.beta, rec.ps, rec.rst);
       arrivals += nblk;
       const bool ok = !any && sync_wait(A.msg, arrivals);
       double v[kSyncBlocks / 32];
@@ -402,12 +410,12 @@ __global__ void __launch_bounds__(kT, 1) k_cg2d_res(const Res32Args A) {
         // 2 beta <p, A p_old> (then <r, A r> < beta^2 <p_old, A p_old>, which
         // CG excludes); the inner solve ends there, its correction so far is
         // kept, and the refinement restarts from the true residual
-        rec.ps = (float)ps;
+        rec.ps = ps;
         // alpha's denominator is <p, A p> less that term: <p, A p> as CG's
         // orthogonality gives it, as in the one-pass kernels (textbook
         // <p, A p> itself let a 512^2 solve without sweeps grow its residual
         // to 1e22 before it stalled)
-        const double den = ps - (double)rec.conj2;
+        const double den = ps - rec.conj2;
         const bool pos = ps > 0.0 && den > 0.0 && finite64(den);
         const double al = pos ? quotient(rec.gm, den) : 0.0;
         const float alf = (float)al;
@@ -530,7 +538,7 @@ __global__ void __launch_bounds__(kT, 1) k_cg2d_res(const Res32Args A) {
           // largest |p|, the test's flag in one word
           sync_put(A.msg, tag, 1, b,
                    __hiloint2double((int)mo, (int)((pm >> 23) << 1 | (any ? 1u : 0u))));
-          sync_put(A.msg, tag, 2, b, __hiloint2double(0, __float_as_int(rs_b)));
+          sync_put(A.msg, tag, 2, b, rs_b);
           sync_put(A.msg, tag, 0, b, sum);
           sync_arrive(A.msg);
         }
@@ -546,25 +554,22 @@ __global__ void __launch_bounds__(kT, 1) k_cg2d_res(const Res32Args A) {
       if (tid == 0) rec.inv_gm = 1.0 / rec.gm;
       arrivals += nblk;
       const bool ok = sync_wait(A.msg, arrivals);
-      double v[kSyncBlocks / 32], v2[kSyncBlocks / 32];
+      asm volatile("bar.arrive 2, 64;" ::: "memory");   // warp 1 goes on
+      double v[kSyncBlocks / 32];
       sync_get(A.msg, tag, 1, nblk, v);
-      sync_get(A.msg, tag, 2, nblk, v2);
       unsigned rm = 0, pmx = 0, fl = 0;
-      float rst = 0.f;
 #pragma unroll
       for (int j = 0; j < kSyncBlocks / 32; ++j) {
         const unsigned lo = (unsigned)__double2loint(v[j]);
         rm = max(rm, (unsigned)__double2hiint(v[j]));
         pmx = max(pmx, (lo >> 1) & 0xffu);
         fl |= lo & 1u;
-        rst += __int_as_float(__double2loint(v2[j]));
       }
       sync_get(A.msg, tag, 0, nblk, v);
       const double G = sync_sum(v);
       rm = __reduce_max_sync(0xffffffffu, rm);
       pmx = __reduce_max_sync(0xffffffffu, pmx);
       fl = __reduce_or_sync(0xffffffffu, fl);
-      for (int o = 16; o > 0; o >>= 1) rst += __shfl_xor_sync(0xffffffffu, rst, o);
       if (tid == 0) {
         const int iter = ++rec.iter, mode = st->mode;
         const float R = __int_as_float((int)rm);
@@ -580,9 +585,12 @@ __global__ void __launch_bounds__(kT, 1) k_cg2d_res(const Res32Args A) {
         const int eg = eb > -1022 ? eb : 0;
         const double gn = eb > -1022 ? __hiloint2double((__double2hiint(G) & 0x800fffff) | 0x3fe00000,
                                                         __double2loint(G)) : G;
-        const float be = ldexpf((float)(gn * rec.inv_gm), eg);
-        // <p, A p_old> = <r_new, A p> + beta <p, A p>
-        rec.conj2 = ldexpf(2.f * be * fmaf(be, rec.ps, rst), -eg);
+        const double bm = gn * rec.inv_gm;   // beta = bm 2^eg
+        const int hb = __double2hiint(bm), xb = (hb >> 20) + eg;
+        const double be = (hb >> 20) > 0 && xb > 0 && xb < 2047
+                              ? __hiloint2double(hb + (eg << 20), __double2loint(bm))
+                              : scalbn(bm, eg);
+        rec.bm = bm;   // (beta in the new units)
         rec.beta = be;
         rec.gm = gn;
         rec.gs += eg;
@@ -595,12 +603,21 @@ __global__ void __launch_bounds__(kT, 1) k_cg2d_res(const Res32Args A) {
           rec.F = F;
           rec.dF = 0;
         }
-        sc.beta = be;
+        sc.beta = (float)be;
         sc.fd = rec.gs - 2 * F;
         sc.thetaF = ldexpf(st->theta, -F);
         sc.check = mode != 0 && (iter & 3) == 3;
         sc.stop = out;
       }
+    }
+    // <r_new, A p> beside it, on an FP64 pipe of its own; needed in the next
+    // exchange only
+    if (wi == 1) {
+      asm volatile("bar.sync 2, 64;" ::: "memory");
+      double v[kSyncBlocks / 32];
+      sync_get(A.msg, tag, 2, nblk, v);
+      const double rst = sync_sum(v);
+      if (lane == 0) rec.rst = rst;
     }
     __syncthreads();
     stop = sc.stop;
@@ -635,7 +652,7 @@ __global__ void __launch_bounds__(kT, 1) k_cg2d_res(const Res32Args A) {
       st->fd = rec.gs - 2 * rec.F;
       st->total_iter += rec.iter - st->iter;
       st->iter = rec.iter;
-      *carry = rec.conj2;
+      *carry = 2.0 * rec.bm * fma(rec.beta, rec.ps, rec.rst);
       if (stop != 0) {
         if (stop == kStall) st->stalled = 1;
         atomicCAS(&st->status, (int)EIK_OK, stop == kStall ? (int)EIK_OK : stop - kStop);
