@@ -138,14 +138,16 @@ __device__ __forceinline__ double sync_sum(const double (&x)[kSyncBlocks / 32]) 
   return s;
 }
 
-// a / b for finite a >= 0 and b > 0 to about one unit in the last place (a
-// step length needs no more): a single-precision reciprocal of b's mantissa
-// and one third-order correction step, y (1 + e + e^2) with e = 1 - m y.  A
-// dependent FP64 operation takes about 90 cycles here; this has five.
+// a / b for finite a >= 0 and b > 0 to within three units in the last place (a
+// step length needs no more): a single-precision reciprocal y of b's mantissa m
+// and the first terms of 1 / m = y / (1 - e) = y (1 + e + e^2 + ...), e = 1 - m y
+// (M. J. Flynn, On division by functional iteration, IEEE Trans. Computers C-19,
+// 1970).  A dependent FP64 operation takes about 90 cycles here; this has five.
 __device__ __forceinline__ double quotient(double a, double b) {
   const int hb = __double2hiint(b);
   const int eb = (hb >> 20) - 1023;
-  if (eb <= -1023 || eb >= 1023) return a / b;   // subnormal or near the top
+  // subnormal (its quotient with a mantissa would be rounded there) or near the top
+  if (eb <= -1023 || eb >= 1023 || (__double2hiint(a) >> 20) == 0) return a / b;
   const double m = __hiloint2double((hb & 0x000fffff) | 0x3ff00000, __double2loint(b));
   const double y = (double)(1.0f / (float)m);
   const double e = fma(-m, y, 1.0);
