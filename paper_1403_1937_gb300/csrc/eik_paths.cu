@@ -115,7 +115,9 @@ __device__ __forceinline__ double dist2(const double *x, const double *y) {
 // below eps.  The square root is monotone, so the test is on the sum itself:
 // t2 is the smallest double whose rounded root is not below eps.  Single
 // precision rules sources out first: with coordinates up to M every |dx| is
-// known to 4 2^-24 M, and the squares to 2^-21 relative.
+// known to 4 2^-24 M, and the squares to 2^-21 relative while they are normal
+// numbers; lim is infinite, which rules nothing out, where t2 is too small for
+// that.
 template <int ND>
 __device__ __forceinline__ bool near_source(const double *x, const double *ys, const float4 *yf,
                                             int nsrc, double t2, float ext, float lim) {
@@ -169,7 +171,9 @@ k_backtrack(Dims3 d, Divisor h, const double *__restrict__ G, const double *__re
       t2 = __longlong_as_double(__double_as_longlong(t2) + 1);
   }
   const bool by_root = !(t2 > 1e-290 && t2 < 1e290);   // eps at the ends of the range
-  const float lim = (float)t2 * 1.0001f;
+  // 1e-30: squares of distances near eps are then normal single-precision
+  // numbers (above 1.2e-38), so that 1e-4 covers their rounding
+  const float lim = (t2 > 1e-30) ? (float)t2 * 1.0001f : INFINITY;
   double x[ND], hi[ND];
 #pragma unroll
   for (int a = 0; a < ND; ++a) {
