@@ -122,12 +122,17 @@ typedef struct {
                          holding the rest as Dirichlet data; 0 = library
                          choice (bands of 40 when the range exceeds 96),
                          negative = never sweep */
-  int test_flags;     /* test hook, 0 in normal use.  Bit 0 (mixed mode): in
-                         the first inner-CG iteration one pipeline (a warp
-                         in 2D, a block in 3D) never gets its first copy,
-                         so its bounded wait (0.2 s) expires and the solve
-                         returns EIK_ERR_TIMEOUT; exercises the timeout path
-                         without any fault. */
+  int test_flags;     /* test hooks, 0 in normal use: a bounded device-side
+                         wait runs out and the solve returns
+                         EIK_ERR_TIMEOUT, without any fault.  Bit 0 (mixed
+                         mode): in the first inner-CG iteration one pipeline
+                         of the one-pass kernels (a warp in 2D, a block in
+                         3D) never gets its first copy (0.2 s); in the
+                         resident 2D kernel one block does not arrive at the
+                         first grid-wide sum (1 s); 3D solves use the
+                         one-pass kernels.  Bit 1 (FP64): likewise in the
+                         first launch of a handle's resident FP64 kernel;
+                         later solves on the handle run as usual. */
   int batch_pack;     /* eik_create_batch of 2D mixed-precision instances:
                          0 (default) or 1 = packed: the instances share one
                          set of FP32 inner-CG arrays and every inner-CG pass

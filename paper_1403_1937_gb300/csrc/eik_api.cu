@@ -296,9 +296,10 @@ eik_status run_cg64(eik_handle *h, double *xs, const double *rhs, const double *
     for (;;) {
       if (h->res.ok) {
         cudaError_t e = cudaSuccess;
+        const bool withhold = (h->opt.test_flags & 2) && h->res.epoch == 0;
         launch_k(h, K_RES64, [&] {
           e = launch_res64(&h->res, h->g, h->sig, xs, h->r, h->p, weight, h->st, h->msg,
-                           h->msg + kSyncBytes / sizeof(*h->msg), h->stream);
+                           h->msg + kSyncBytes / sizeof(*h->msg), withhold, h->stream);
         });
         if (e == cudaErrorCooperativeLaunchTooLarge) {
           // fewer SMs than the device reports (a partitioned context): the

@@ -56,6 +56,7 @@ struct Res64Args {
   unsigned long long *msg, *inbox;
   unsigned epoch;
   int max_it;
+  int withhold;   // test hook: block 0 does not arrive in the first exchange
 };
 
 // Shared-memory layout (doubles first).
@@ -298,7 +299,7 @@ __global__ void __launch_bounds__(kT, 1) k_cg64_res(const Res64Args A) {
     ++tag;
     if (tid < 32) {
       // (a block whose halo never came does not arrive, so every block stops)
-      if (tid == 0 && !any) {
+      if (tid == 0 && !any && !(A.withhold && it == 0 && b == 0)) {
         sync_put(A.msg, tag, 0, b, s);
         sync_arrive(A.msg);
       }
@@ -534,8 +535,10 @@ void res64_plan(Res64Plan *pl, const Grid &g, int num_sms) {
 
 cudaError_t launch_res64(Res64Plan *pl, const Grid &g, const double *sig, double *x, double *r,
                          double *p, const double *cw_weight, CgState *st,
-                         unsigned long long *msg, unsigned long long *inbox, cudaStream_t s) {
+                         unsigned long long *msg, unsigned long long *inbox, bool withhold,
+                         cudaStream_t s) {
   Res64Args a{};
+  a.withhold = withhold ? 1 : 0;
   a.g = g;
   a.cx = pl->cx;
   a.cy = pl->cy;

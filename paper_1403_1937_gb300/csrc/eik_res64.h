@@ -24,9 +24,11 @@ void res64_plan(Res64Plan *pl, const Grid &g, int num_sms);
 // Runs up to a few hundred CG iterations from (x, r, p) and *st, as the two
 // passes of eik_cg64.cu do, and writes them back.  msg: the solver's message
 // buffer (kSyncBytes) and inbox the halo buffer (inbox_words), both zeroed
-// when they were allocated.
+// when they were allocated.  withhold: test hook, one block does not arrive in
+// the launch's first grid-wide sum, so that the waits run out (EIK_ERR_TIMEOUT).
 cudaError_t launch_res64(Res64Plan *pl, const Grid &g, const double *sig, double *x, double *r,
                          double *p, const double *cw_weight, CgState *st,
-                         unsigned long long *msg, unsigned long long *inbox, cudaStream_t s);
+                         unsigned long long *msg, unsigned long long *inbox, bool withhold,
+                         cudaStream_t s);
 
 }  // namespace eik
