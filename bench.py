@@ -44,9 +44,8 @@ ALGO_BYTES_PER_NODE = {
     "cg_pass2_64": 56,   # read x, r, p, q; write x, r, p     (7 x 8 B)
     # one single-reduction FP32 inner iteration: read r, p, sig, d; write r,
     # p (other buffer set) and d (7 x 4 B); the checking passes (every 4th
-    # in later refinement steps) also read the FP32 iterate, not counted
-    # (the two-pass 3D kernels move 11 words, the resident 2D ones d at most;
-    # their times are per iteration, and the same 7 words are counted)
+    # in later refinement steps) also read the FP32 iterate, not counted.  The
+    # one-pass kernels' figure; see inner_cg_bytes for the others
     "mixed_cg": 28,
     "mixed_cg_init": 8,  # first pass of an inner solve: read r, sig
     # FP64 residual of a refinement step: read sig, x (f64); write r, p, d,
@@ -71,6 +70,18 @@ def algo_bytes(kernel, inst):
     if kernel == "mixed_mg" and len(inst.dims) == 3:
         return 85
     return ALGO_BYTES_PER_NODE[kernel]
+
+
+def inner_cg_bytes(kernel_ms, inst):
+    """Bytes per node and iteration of the inner-CG kernels that a solve ran
+    (all report as mixed_cg, timed by iterations).  The one-pass kernels, which
+    have a timed first pass: 28.  The two-pass 3D kernels: read r, p_old, sig,
+    write p, q; read p, q, d, r, write d, r: 44.  The resident 2D kernel keeps r,
+    p and sigma on chip: None."""
+    if kernel_ms.get("mixed_cg_init", (None,))[0] is not None:
+        return ALGO_BYTES_PER_NODE["mixed_cg"]
+    return 44 if len(inst.dims) == 3 else None
+
 
 # The FP64 passes are bound by the FP64 pipe, not by HBM: their roofline is
 # algorithmic FP64 operations (an FMA counts 2) per node against the GB300's
@@ -405,6 +416,9 @@ def measure(args, wname, ws, local, modes=None):
         eik.eik_solve(hd, S_out=S_dev)
         eik.eik_set_profiling(hd, False)
         prof = eik.eik_kernel_stats(hd)
+        if not prof.get("mixed_cg_init", (0, 0))[1]:
+            # inner solves that began without a launch of their own
+            res["gpu_launches"] -= kst.get("mixed_cg_init", (0,))[0]
         res["kernel_ms"] = {k: (v[2] / v[1] if v[1] else None, v[1], v[2])
                             for k, v in prof.items() if v[0]}
         results[mode] = res
@@ -422,8 +436,10 @@ def kernel_table(res, inst):
         if avg_ms is None:
             continue
         e = {"avg_us": round(avg_ms * 1e3, 2), "timed_launches": n}
-        if k in ALGO_BYTES_PER_NODE:
-            gbs = algo_bytes(k, inst) * inst.n / (avg_ms * 1e-3) / 1e9
+        per_node = (inner_cg_bytes(res["kernel_ms"], inst) if k == "mixed_cg"
+                    else algo_bytes(k, inst) if k in ALGO_BYTES_PER_NODE else None)
+        if per_node is not None:
+            gbs = per_node * inst.n / (avg_ms * 1e-3) / 1e9
             e["achieved_gbs"] = round(gbs, 1)
             e["frac_of_hbm"] = round(gbs / peak, 4)
         out[k] = e
@@ -648,9 +664,10 @@ def run_batch(args, emit=True):
 def fft_flops(n, terms):
     """FP64 operations of the 1D transforms eik_fft_series runs on an n x n
     grid with `terms` terms, at the usual 5 N log2 N per complex transform of
-    length N: transform length P = the smallest 2^a 3^b 5^c >= 2n - 1; the
-    kernels' transforms (G~, and G when terms > 0) take 2P row transforms, a
-    grid function's forward transform n + P and its inverse P + n."""
+    length N: transform length P = the smallest 2^a 3^b 5^c >= 2n - 1, of which
+    H = P / 2 + 1 columns are kept.  Two real rows share one transform: a grid
+    function takes (n + 1) / 2 row and H column transforms each way, a kernel
+    (G~, and G when terms > 0), even in both axes, (n + 1) / 2 + (H + 1) / 2."""
     P = max(2 * n - 1, 2)
     while True:
         q = P
@@ -661,8 +678,9 @@ def fft_flops(n, terms):
             break
         P += 1
     per = 5 * P * np.log2(P)
-    kernels = 2 * P * (1 + (1 if terms > 0 else 0))
-    data = (1 + terms) * 2 * (n + P)
+    H, pairs = P // 2 + 1, (n + 1) // 2
+    kernels = (pairs + (H + 1) // 2) * (1 + (1 if terms > 0 else 0))
+    data = (1 + terms) * 2 * (pairs + H)
     return float(per * (kernels + data))
 
 
@@ -717,7 +735,8 @@ def run_fft(args):
             "config": {"workload": "Sec. 5.4 Example 1: f = exp(r) on [-0.125, 0.125]^2, "
                                    "one source at the origin, 6 terms",
                        "grids": rows},
-            "roofline": {"bound": "fp64", "kernel": "k_fft_rows (all transforms)",
+            "roofline": {"bound": "fp64", "kernel": "k_rows_x, k_cols, k_kernel_rows, "
+                                                   "k_kernel_cols (all transforms)",
                          "achieved": rows[-1]["transform_tflops"], "peak": peak,
                          "unit": "TFLOP/s",
                          "frac": round(rows[-1]["transform_tflops"] / peak, 4),
@@ -853,11 +872,20 @@ def roofline(res, inst, wname, only=None):
                 "algorithmic_bytes_per_launch": ALGO_BYTES_PER_NODE[dom] * inst.n,
                 "avg_launch_ms": avg_ms,
                 "share_of_kernel_time": round(cand[dom][2] / total, 3) if total else None}
-    algo = algo_bytes(dom, inst) * inst.n
+    per_node = inner_cg_bytes(km, inst) if dom == "mixed_cg" else algo_bytes(dom, inst)
+    if per_node is None:
+        return {"bound": "on-chip", "kernel": dom, "frac": None,
+                "note": "k_cg2d_res: r, p and sigma stay in registers and shared memory, and d stays in L2 or "
+                        "registers, so no share of the HBM bandwidth is stated; an iteration is "
+                        "the tile's arithmetic, its spills and two grid-wide sums",
+                "achieved": round(1e3 * avg_ms, 2), "peak": None, "unit": "us/iteration",
+                "traffic": None, "avg_launch_ms": avg_ms,
+                "share_of_kernel_time": round(cand[dom][2] / total, 3) if total else None}
+    algo = per_node * inst.n
     achieved = algo / (avg_ms * 1e-3) / 1e9
-    # the recorded inner-CG counters are the one-pass kernels', which have a
-    # first pass of their own (the resident and the two-pass kernels have none)
-    traffic = (ncu_traffic(dom, wname) if dom != "mixed_cg" or "mixed_cg_init" in km else None)
+    # the recorded inner-CG counters are the one-pass kernels'
+    traffic = (ncu_traffic(dom, wname)
+               if dom != "mixed_cg" or per_node == ALGO_BYTES_PER_NODE["mixed_cg"] else None)
     return {"bound": "hbm", "kernel": dom, "achieved": round(achieved, 1),
             "peak": peak, "peak_source": peak_src, "unit": "GB/s",
             "frac": round(achieved / peak, 4), "traffic": traffic,
