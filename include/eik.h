@@ -102,14 +102,19 @@ typedef struct {
   int boundary;       /* EIK_BOUNDARY_*; default half cell */
   int tile_override;  /* mixed-mode inner-CG kernel variant (results agree
                          to rounding; for tuning and tests):
-                         0 = library choice (variant 1);
+                         0 = library choice: in 2D the resident kernel where
+                         the grid fits on chip, in 3D the two-pass kernels
+                         (two sums an iteration; last refinement steps aim
+                         at tol / 8), variant 1 elsewhere, and beyond 96
+                         powers of two of phi in one inner solve;
+                         1..4 = one-pass kernels (one sum an iteration; last
+                         steps aim at tol / 2):
                          2D (every warp an independent pipeline over tiles
-                         of 128 columns): 1..4 = (row stages per warp,
-                         warps per block) = (5, 5), (6, 4), (7, 4), (6, 7);
+                         of 128 columns): (row stages per warp, warps per
+                         block) = (5, 5), (6, 4), (7, 4), (6, 7);
                          3D (a block marches 128 x TY rows through z):
-                         1..4 = (TY, plane stages) = (12, 5), (8, 6),
-                         (16, 4), (8, 8).  Other values return
-                         EIK_ERR_ARG. */
+                         (TY, plane stages) = (12, 5), (8, 6), (16, 4),
+                         (8, 8).  Other values return EIK_ERR_ARG. */
   double inner_tol;   /* mixed mode: factor by which the first FP32 inner
                          solve of a refinement step reduces the residual
                          (scaled max norm); 0 = library choice (1e-1) */
@@ -399,10 +404,14 @@ eik_status eik_fft_series(const int64_t *dims, double h, double hbar, const doub
 /* Per-kernel counters of a handle (diagnostics; the paper has no
  * counterpart).  launches counts every kernel launch the handle issued since
  * creation or the last eik_reset_kernel_stats (kernels inside captured graphs
- * count once per graph launch).  total_ms is the summed device time of those
- * launches measured with CUDA events on the library's stream; it is filled
- * only for launches made while profiling is enabled (eik_set_profiling),
- * which replaces graph launches by individually timed launches. */
+ * count once per graph launch).  mixed_cg_init counts the inner solves begun:
+ * in the one-pass kernels a launch each, while the resident and the two-pass
+ * kernels begin without one (its timed_launches are launches in any case).
+ * total_ms is the summed device time of the timed launches, measured with CUDA
+ * events on the library's stream; it is filled only for launches made while
+ * profiling is enabled (eik_set_profiling), which replaces graph launches by
+ * individually timed launches.  mixed_cg is timed by iterations: its
+ * timed_launches are iterations and total_ms their time. */
 typedef struct {
   char name[32];
   int64_t launches;

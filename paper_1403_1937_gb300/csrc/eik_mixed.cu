@@ -862,8 +862,8 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
         for (auto &e : m->ev) MCK(cudaEventCreate(&e));
       if (m->profile) MCK(cudaEventRecord(m->ev[0], s));
       // (the resident and the two-pass kernels start from the residual's
-      // <r, r>; they have no initial pass, and the count below is of inner
-      // solves)
+      // <r, r>; they have no initial pass, and the count below, reported as
+      // mixed_cg_init, is of inner solves)
       const bool init = !m->use_res && !m->use_pair;
       const int per_iter = m->use_pair ? 2 : 1;   // launches
       if (init) cg32_init(m->plan, g, m->cg, m->bufs, 0, s);
