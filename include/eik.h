@@ -119,7 +119,11 @@ typedef struct {
                          solve of a refinement step reduces the residual
                          (scaled max norm); 0 = library choice (1e-1) */
   int max_outer;      /* mixed mode: refinement steps (per level-set band);
-                         0 = library choice (30) */
+                         0 = library choice (30).  A solve that does not
+                         converge with the resident or the two-pass kernels
+                         starts again with the one-pass kernels (see
+                         tile_override) and the same limit, within what is
+                         left of max_iter. */
   int band_bits;      /* mixed mode: when the coarse distance estimate puts
                          phi over more than 2 * band_bits powers of two, the
                          solve sweeps level-set bands of band_bits powers of

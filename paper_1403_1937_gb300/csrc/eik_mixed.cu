@@ -793,13 +793,16 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
     // (cw is infinite while some node of the iterate is not positive yet;
     // progress is then judged only once it is finite)
     // a step that recovers from a bad correction (an inner solve that lost
-    // conjugacy late) counts as progress too
+    // conjugacy late) counts as progress too: without it solves over 90 powers of
+    // two were given up that the next steps finish
     const bool recovering = cw < 0.5 * last_cw;
     last_cw = cw;
     if (!std::isfinite(cw) || cw < 0.5 * best_cw) {
       if (std::isfinite(cw)) best_cw = cw;
       stall = 0;
-    } else if (again == kMgFirst && !recovering && ++stall >= 2) {
+    } else if (recovering) {
+      stall = 0;
+    } else if (again == kMgFirst && ++stall >= 2) {
       g_msg = "mixed refinement stopped making progress";
       break;
     }
@@ -946,9 +949,11 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
   return result;
 }
 
-eik_status mixed_solve(MixedState *m, const MixedArgs &a, int *inner_iters, int *outer_iters,
-                       double *res_cw, double *res_nw) {
-  static const bool trace = getenv("EIK_TRACE_MIXED") != nullptr;
+// The whole solve from the zero iterate.  *two_sum: whether the two-sum kernels
+// may run; returns whether they did.  Iterations and steps are added to
+// *inner_iters and *outer_iters.
+static eik_status solve_once(MixedState *m, const MixedArgs &a, bool *two_sum, int *inner_iters,
+                             int *outer_iters, double *res_cw, bool trace) {
   const Grid &g = m->g;
   cudaStream_t s = a.stream;
   const int cap = m->cap;
@@ -994,14 +999,17 @@ eik_status mixed_solve(MixedState *m, const MixedArgs &a, int *inner_iters, int 
   // where the two-sum one may not (512^2, hbar = 2.6 h, no sweeps: its
   // residual grew from step to step).  The test hook withholds a copy of the
   // one-pass kernels in 3D.
+  const bool allowed = *two_sum;
+  *two_sum = false;
   auto pick_kernels = [&](int span) -> eik_status {
     if (m->batch || m->mg) return EIK_OK;
-    m->use_res = m->res.ok && span <= kSweepBits;
-    m->use_pair = m->pair.ok && span <= kSweepBits && !(a.opt.test_flags & 1);
+    m->use_res = allowed && m->res.ok && span <= kSweepBits;
+    m->use_pair = allowed && m->pair.ok && span <= kSweepBits && !(a.opt.test_flags & 1);
+    *two_sum = *two_sum || m->use_res || m->use_pair;
     return m->use_res ? EIK_OK : build_graph(m, s);
   };
   const int max_outer = (a.opt.max_outer > 0) ? a.opt.max_outer : 30;
-  int total = 0, outer = 0;
+  int &total = *inner_iters, &outer = *outer_iters;
   eik_status result;
   const int sweep_bits = (a.opt.band_bits > 0) ? 2 * a.opt.band_bits
                                                : (m->mg ? kMgSweepBits : kSweepBits);
@@ -1052,10 +1060,26 @@ eik_status mixed_solve(MixedState *m, const MixedArgs &a, int *inner_iters, int 
     }
     if (result == EIK_ERR_NOT_CONVERGED) g_msg = "level-set sweeps did not converge";
   }
-  *inner_iters = total;
-  *outer_iters = outer;
-  *res_nw = 0.0;
   return result;
+}
+
+eik_status mixed_solve(MixedState *m, const MixedArgs &a, int *inner_iters, int *outer_iters,
+                       double *res_cw, double *res_nw) {
+  static const bool trace = getenv("EIK_TRACE_MIXED") != nullptr;
+  *inner_iters = *outer_iters = 0;
+  *res_nw = 0.0;
+  bool two_sum = true;
+  eik_status st = solve_once(m, a, &two_sum, inner_iters, outer_iters, res_cw, trace);
+  // Where the two-sum kernels' inner solves come apart too often, the solve
+  // starts again with the one-pass kernels, within what is left of the
+  // iterations (2 of 1,100 drawn 2D fields with phi over 20 to 400 powers of two)
+  if (two_sum && *inner_iters < a.opt.max_iter &&
+      (st == EIK_ERR_NOT_CONVERGED || st == EIK_ERR_BREAKDOWN)) {
+    if (trace) fprintf(stderr, "[mixed] again with the one-pass kernels\n");
+    two_sum = false;
+    st = solve_once(m, a, &two_sum, inner_iters, outer_iters, res_cw, trace);
+  }
+  return st;
 }
 
 eik_status mixed_export_hat(MixedState *m, const MixedArgs &a, double *xh) {
