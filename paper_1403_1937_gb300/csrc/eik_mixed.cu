@@ -830,8 +830,9 @@ static eik_status refine(MixedState *m, const MixedArgs &a, int lo, int hi, int 
     st.thresh = (float)(red * st.r_inf);
     // a step whose aim is below tol is probably the last one: the two-sum
     // kernels then go to tol / 8 (on eight grids at tol 1e-6 and 1e-8: 2 % more
-    // iterations, S up to 12 times nearer; at tol / 2 a 2048^2 solve to 1e-6
-    // ended at cw = 9.6e-7 with S off by 1.1e-6, at tol / 8 by 1.5e-7)
+    // iterations, S up to 12 times nearer; at tol 1e-9, close to what FP32 steps
+    // reach, up to 25 % more; at tol / 2 a 2048^2 solve to 1e-6 ended at cw =
+    // 9.6e-7 with S off by 1.1e-6, at tol / 8 by 1.5e-7)
     const double aim = 1e-3 * cw;
     st.theta = (float)(aim < tol && (m->use_res || m->use_pair) ? 0.125 * tol
                                                               : std::max(0.5 * tol, aim));
